@@ -183,9 +183,9 @@ __device__ __forceinline__ void init_m(const DevInstance& in, const DevSolve& s,
 
 // Sign-round, outputs and the replica's energy (pairs a < b once plus the
 // field). The lanes stride along row a, so every load of the row is
-// coalesced; integer J sums exactly in int64, and for other couplings the
-// library re-evaluates this sum exactly afterwards when the instance's span
-// allows it.
+// coalesced; integer J sums exactly in int64. With skip_energy the library
+// evaluates the energies exactly afterwards (launch_energy) and none is summed
+// here.
 __device__ void finish_replica(const DevInstance& in, const DevSolve& s, int r, const float* m,
                                int lane, const Level& lv)
 {
@@ -197,7 +197,7 @@ __device__ void finish_replica(const DevInstance& in, const DevSolve& s, int r, 
     }
     long long ei = 0;
     double ef = 0.0;
-    for (int a = 0; a < n; ++a) {
+    for (int a = 0; a < n && !s.skip_energy; ++a) {
         const int sa = m[a] >= 0.f ? 1 : -1;
         if (in.integer) {
             const int8_t* row = in.J_i8 + (size_t)a * n;

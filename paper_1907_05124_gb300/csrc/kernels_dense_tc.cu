@@ -974,7 +974,9 @@ __global__ void tc_compact_gather_kernel(TcState t, const int32_t* rep, TcCompac
     }
 }
 
-// Sign-round, outputs in caller labels and exact energy, one CTA per slot.
+// Sign-round and outputs in caller labels, one CTA per slot, and the energies
+// that no launch_energy follows for (energy_pass): small integer instances, in
+// int64, and couplings whose span exceeds the exact accumulator, in FP64.
 __global__ void __launch_bounds__(256) tc_finalize_kernel(TcState t, DevInstance in, DevSolve s)
 {
     __shared__ long long s_i[8];
@@ -990,6 +992,7 @@ __global__ void __launch_bounds__(256) tc_finalize_kernel(TcState t, DevInstance
         const int o = __ldg(in.new2old + a);
         s.sigma[(size_t)r * n + o] = (int8_t)sa;
         if (s.m_final) s.m_final[(size_t)r * n + o] = m[a];
+        if (s.skip_energy) continue;
         if (in.integer) {
             const int8_t* row = in.J_i8 + (size_t)a * n;
             int acc = 0;

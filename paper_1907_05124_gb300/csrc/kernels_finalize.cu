@@ -38,7 +38,8 @@ __global__ void __launch_bounds__(kBestThreads) best_kernel(DevSolve s, int32_t 
 
 constexpr int kEnergyThreads = 256;
 
-// Energies of spin vectors, one CTA per vector. Integer couplings sum exactly
+// Energies of spin vectors, one CTA per vector: sparse instances, and dense
+// ones whose span exceeds the exact accumulator. Integer couplings sum exactly
 // in int64; other couplings sum exactly in an ExactAcc and are rounded once.
 __global__ void __launch_bounds__(kEnergyThreads) energy_kernel(DevInstance in, const int8_t* spins,
                                                                 double* e, long long* e_i64,
@@ -58,19 +59,9 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_kernel(DevInstance in, 
     for (int a = tid; a < n; a += kEnergyThreads) {
         const int sa = sp[__ldg(in.new2old + a)];
         if (sa != 1 && sa != -1) { atomicExch(status, (int)kDevBadIndex); continue; }
-        if (in.dense) {
-            if (in.integer) {
-                const int8_t* row = in.J_i8 + (size_t)a * n;
-                long long acc = 0;
-                for (int b = a + 1; b < n; ++b) acc += (int)row[b] * (int)sp[__ldg(in.new2old + b)];
-                ei += acc * sa;
-            } else {
-                const double* row = in.J_f64 + (size_t)a * n;
-                for (int b = a + 1; b < n; ++b) {
-                    const double w = sa * sp[__ldg(in.new2old + b)] > 0 ? row[b] : -row[b];
-                    if (exact) ex.add(w, in.exact_e0); else ef += w;
-                }
-            }
+        if (in.dense) {  // the span exceeds the accumulator (launch_energy)
+            const double* row = in.J_f64 + (size_t)a * n;
+            for (int b = a + 1; b < n; ++b) ef += sa * sp[__ldg(in.new2old + b)] > 0 ? row[b] : -row[b];
         } else {
             const int e0 = __ldg(in.row_ptr + a), e1 = __ldg(in.row_ptr + a + 1);
             if (in.integer) {
@@ -167,6 +158,7 @@ cudaError_t launch_energy(const DevInstance& in, const int8_t* spins, int32_t co
                           long long* e_i64, int32_t* status, cudaStream_t st)
 {
     if (count <= 0) return cudaSuccess;
+    if (in.dense && (in.integer || in.exact_ok)) return launch_dense_energy(in, spins, count, e, e_i64, status, st);
     energy_kernel<<<count, kEnergyThreads, 0, st>>>(in, spins, e, e_i64, status);
     return cudaGetLastError();
 }

@@ -244,6 +244,7 @@ void exact_span(const std::vector<double>& vals, const std::vector<double>& h, i
     int grow = 0;
     while ((int64_t)1 << grow < terms + 1 && grow < 62) ++grow;
     d->exact_e0 = lo;
+    d->exact_bits = hi - lo;
     d->exact_ok = (hi + grow - lo) <= 220 && lo >= -1126;
 }
 
@@ -497,6 +498,8 @@ int mars_instance_dense(mars_ctx* c, int32_t n, const void* J, int32_t jt, const
     d.nlev = n;
     d.integer = integer;
     d.n_pad = n_pad;
+    d.identity = 1;
+    for (int32_t a = 0; a < n; ++a) d.identity &= o[a] == a;
     if (!integer) exact_span(Jh, hh, (int64_t)n * (n - 1) / 2 + n, &d);
     {
         const uint16_t* jb = nullptr;
@@ -845,6 +848,7 @@ int mars_solve(mars_ctx* c, int32_t id, const mars_params* p, int8_t* best_spins
     set_schedule(s, p);
     s.jacobi = p->update == MARS_UPDATE_JACOBI;
     set_method(s, p);
+    s.skip_energy = in->dev.dense && energy_pass(in->dev, tc, R);
     // start temperatures
     float* t0 = nullptr;
     if ((rc = S.get(R, &t0))) return rc;
@@ -977,8 +981,8 @@ int mars_solve(mars_ctx* c, int32_t id, const mars_params* p, int8_t* best_spins
         ++launches;
     }
     launches += tcprof.launches;
-    if (!in->dev.integer && in->dev.exact_ok) {  // replace the kernels' FP64 sums by exact ones
-        MARS_CUDA(c, launch_energy(in->dev, s.sigma, R, s.energy, nullptr, s.status, st));
+    if (energy_pass(in->dev, tc, R)) {
+        MARS_CUDA(c, launch_energy(in->dev, s.sigma, R, s.energy, s.energy_i64, s.status, st));
         ++launches;
     }
     MARS_CUDA(c, cudaEventRecord(c->ev2, st));
@@ -1155,7 +1159,7 @@ int mars_solve_batch(mars_ctx* c, int32_t count, const int32_t* insts, const mar
     ++launches;
     for (int32_t j = 0; j < count; ++j) {
         const DevSolve& s = jobs[j].s;
-        if (!dins[j].integer && dins[j].exact_ok) {
+        if (energy_pass(dins[j], false, jobs[j].s.R)) {
             MARS_CUDA(c, launch_energy(dins[j], s.sigma, s.R, s.energy, nullptr, s.status, st));
             ++launches;
         }

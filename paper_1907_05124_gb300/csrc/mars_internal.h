@@ -59,11 +59,13 @@ struct DevInstance {
     // term is a multiple of 2^exact_e0 and every sum fits the accumulator
     int32_t exact_ok = 0;
     int32_t exact_e0 = 0;
+    int32_t exact_bits = 0;            // every |term| is below 2^(exact_e0 + exact_bits)
     // common
     const float* h = nullptr;          // n floats or null
     const double* h_f64 = nullptr;     // n doubles or null
     const float* inv_norm = nullptr;   // n: 1 / sqrt(h_i^2 + sum_j J_ij^2), 0 where that is 0 (NMFA)
     const int32_t* new2old = nullptr;  // n
+    int32_t identity = 0;              // new labels are the caller's (new2old[a] = a)
 };
 
 struct DevResult {
@@ -103,6 +105,7 @@ struct DevSolve {
     float nmfa_alpha = 0.5f, nmfa_sigma = 0.f;
     const double* t_first = nullptr;   // optional per-replica temperature of the first level
     int32_t one_level = 0;             // stop after the first level (the FP32 polish)
+    int32_t skip_energy = 0;           // the dense kernels leave the energies to launch_energy
     int32_t add_counts = 0;            // add sweeps/levels/capped to the outputs' values
     float* m_scratch = nullptr;        // per-CTA state when it does not fit on chip
     float* m_next = nullptr;           // per-CTA second buffer for synchronous sweeps
@@ -379,6 +382,22 @@ cudaError_t launch_flag_wait(const int32_t* flag, long long budget_cycles, int32
 cudaError_t launch_best(const DevSolve& s, int32_t n, int32_t integer, int8_t* best_spins,
                         DevResult* res, cudaStream_t st);
 
+// Whether the energies of a solve of R replicas come from launch_energy after
+// the descent: the exact sums of non-integer couplings, and dense integer
+// instances on the tensor-core path (`tc`) once the tiled pass beats the
+// finalize kernel's own sums. Those cost about 6e-13 s R n^2 on a GB300 (n =
+// 8192, R = 4096: 163 ms; the pass 5.7) and a serial walk along each row; the
+// pass never takes less than about 40 us.
+inline bool energy_pass(const DevInstance& in, bool tc, int32_t R)
+{
+    if (!in.integer) return in.exact_ok != 0;
+    return in.dense && tc && (in.n > 512 || (double)R * in.n * in.n > 6.6e7);
+}
+
+// Exact energies of dense instances with integer couplings or exact_ok
+// (kernels_dense_energy.cu); launch_energy routes them here.
+cudaError_t launch_dense_energy(const DevInstance& in, const int8_t* spins, int32_t count, double* e,
+                                long long* e_i64, int32_t* status, cudaStream_t st);
 cudaError_t launch_energy(const DevInstance& in, const int8_t* spins, int32_t count,
                           double* e, long long* e_i64, int32_t* status, cudaStream_t st);
 

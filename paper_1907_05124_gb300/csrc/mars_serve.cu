@@ -290,8 +290,8 @@ int serve_copy_results(mars_ctx* c, ServeReq* q)
 int serve_finish_enqueue(mars_ctx* c, ServeReq* q)
 {
     cudaStream_t st = q->st;
-    if (!q->dev.integer && q->dev.exact_ok)
-        MARS_CUDA(c, launch_energy(q->dev, q->s.sigma, q->s.R, q->s.energy, nullptr, q->s.status, st));
+    if (energy_pass(q->dev, q->tc != nullptr, q->s.R))
+        MARS_CUDA(c, launch_energy(q->dev, q->s.sigma, q->s.R, q->s.energy, q->s.energy_i64, q->s.status, st));
     MARS_CUDA(c, launch_best(q->s, q->dev.n, q->dev.integer, q->dbest, q->dres, st));
     return serve_copy_results(c, q);
 }
@@ -347,6 +347,8 @@ int serve_launch(mars_ctx* c, Serve* sv, ServeReq* q)
     set_schedule(s, &p);
     s.jacobi = p.update == MARS_UPDATE_JACOBI;
     set_method(s, &p);
+    s.skip_energy =
+        q->dev.dense && energy_pass(q->dev, p.precision == MARS_BF16 || p.precision == MARS_FP8, R);
     s.m0 = p.m0;
     float* t0 = nullptr;
     if ((rc = get((size_t)R * sizeof(float), (void**)&t0))) return rc;
