@@ -323,6 +323,13 @@ cudaError_t launch_tc_pair_gemm(const CUtensorMap& tmJ, const CUtensorMap& tmS, 
 // active replicas spread over more SMs); the per-replica arithmetic is the same.
 cudaError_t launch_tc_chain(const TcState& t, int p, int rpw, int cw, const float* G, const float* gx_in,
                             float* gx_out, bool g_early, cudaStream_t st);
+// The same chain with its sequential steps on one warp per CTA and the folds on
+// others (kernels_dense_chain.cu), for rpc (8, 16 or 32) replica slots per
+// CTA; bit for bit the results of launch_tc_chain.
+cudaError_t launch_tc_split_chain(const TcState& t, int p, int rpc, const float* G, const float* gx_in,
+                                  float* gx_out, bool g_early, cudaStream_t st);
+// Launch with programmatic stream serialization (kernels_dense_tc.cu).
+cudaError_t launch_pdl(const void* k, dim3 grid, dim3 block, void** args, size_t smem, cudaStream_t st);
 // Compaction of the active replicas into the first slots: scratch of the
 // same shapes as TcState's per-slot arrays (rows of n_pad spins for S and its
 // low-precision copy) and the permutation.

@@ -149,7 +149,22 @@ int tc_plan(mars_ctx* c, TcRun* run, int32_t active, int32_t prefix)
     // crowd out the GEMM (1024 active: 12.8 against 18.1 us per panel).
     int cw = (chain_slots + 4 * rpw - 1) / (4 * rpw) <= run->sms / 2 ? 4 : 8;
     if (const int f = env_flag("MARS_TC_CHAIN_WARPS", 0); f == 4 || f == 8) cw = f;
-    if (run->exec && rpw == run->rpw && ovl == run->overlap && pr == run->pair && splitk == run->splitk &&
+    // Beyond that the split chain (launch_tc_split_chain), with as few replica
+    // slots per CTA as leave the SMs of one wave to it and, with the overlap,
+    // to the GEMM beside it. One sweep at N = 8192, ms, chain_body's kernel
+    // against 8 / 16 / 32 slots: 512 active 0.74, 0.66 / 0.75 / 1.03; 1024
+    // 0.99, 1.26 / 0.78 / 0.93; 1400 1.27, 1.33 / 1.24 / 0.94; 2048 1.49,
+    // 1.36 / 1.10 / 1.18; 4096 1.96, 2.46 / 1.94 / 1.47. With 128 active (4
+    // warps) 0.61 against 0.64: the step's latency bounds both, and the split
+    // chain hands its fields over twice.
+    int rpc = 0;
+    if (cw != 4 && run->fixed_rpw < 0 && env_flag("MARS_TC_CHAIN_WARPS", 0) == 0) {
+        const int free_sms = ovl ? run->sms - tiles * splitk : run->sms;
+        rpc = 8;
+        while (rpc < 32 && (chain_slots + rpc - 1) / rpc > free_sms) rpc *= 2;
+    }
+    if (const int v = env_flag("MARS_TC_CHAIN_RPC", -1); v == 0 || v == 8 || v == 16 || v == 32) rpc = v;
+    if (run->exec && rpc == run->chain_rpc && rpw == run->rpw && ovl == run->overlap && pr == run->pair && splitk == run->splitk &&
         tiles == run->gemm_tiles && chain_slots == run->chain_slots && cw == run->chain_warps)
         return MARS_OK;
     if (run->exec) cudaGraphExecDestroy(run->exec);
@@ -158,6 +173,7 @@ int tc_plan(mars_ctx* c, TcRun* run, int32_t active, int32_t prefix)
     run->graph = nullptr;
     run->rpw = rpw;
     run->chain_warps = cw;
+    run->chain_rpc = rpc;
     run->overlap = ovl;
     run->pair = pr;
     run->splitk = splitk;
@@ -291,6 +307,10 @@ int tc_enqueue_sweep(mars_ctx* c, TcRun* run, cudaStream_t st, bool timed)
     // the chains cover the slots below the active prefix the plan was made for
     TcState tc = run->t;
     tc.R = run->chain_slots;
+    auto chain = [&](int p, const float* G, const float* gx_in, float* gx_out, bool g_early) {
+        return run->chain_rpc ? launch_tc_split_chain(tc, p, run->chain_rpc, G, gx_in, gx_out, g_early, st)
+                              : launch_tc_chain(tc, p, run->rpw, run->chain_warps, G, gx_in, gx_out, g_early, st);
+    };
     if (run->pair) {
         // panels in pairs: one GEMM for panels pp and pp+1, chain pp (which
         // adds its new spins to panel pp+1's fields), chain pp+1
@@ -316,10 +336,9 @@ int tc_enqueue_sweep(mars_ctx* c, TcRun* run, cudaStream_t st, bool timed)
             }
             // chain pp's fields come from the GEMM just before it; chain pp+1's
             // from the same GEMM, two kernels back
-            MARS_CUDA(c, launch_tc_chain(tc, pp, run->rpw, run->chain_warps, run->Gbuf[0], nullptr, two ? run->Gx[0] : nullptr,
-                                         false, st));
+            MARS_CUDA(c, chain(pp, run->Gbuf[0], nullptr, two ? run->Gx[0] : nullptr, false));
             if (two)
-                MARS_CUDA(c, launch_tc_chain(tc, pp + 1, run->rpw, run->chain_warps, run->Gbuf[1], run->Gx[0], nullptr, true, st));
+                MARS_CUDA(c, chain(pp + 1, run->Gbuf[1], run->Gx[0], nullptr, true));
         }
         MARS_CUDA(c, launch_tc_advance(run->t, st));
         return MARS_OK;
@@ -349,7 +368,7 @@ int tc_enqueue_sweep(mars_ctx* c, TcRun* run, cudaStream_t st, bool timed)
         float* gx_out = ov && pp + 1 < P ? run->Gx[(pp + 1) & 1] : nullptr;
         // the GEMM's event edge into the chain may be captured as a
         // programmatic edge too, so its fields are read after the wait
-        MARS_CUDA(c, launch_tc_chain(tc, pp, run->rpw, run->chain_warps, run->Gbuf[pp & 1], gx_in, gx_out, false, st));
+        MARS_CUDA(c, chain(pp, run->Gbuf[pp & 1], gx_in, gx_out, false));
         if (ov) MARS_CUDA(c, cudaEventRecord(run->ev[2 + 2 * pp], st));
     }
     MARS_CUDA(c, launch_tc_advance(run->t, st));

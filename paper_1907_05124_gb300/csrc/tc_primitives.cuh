@@ -60,12 +60,48 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity)
     return ok != 0;
 }
 
+// Whether the phase with the given parity has completed, without waiting
+// (try_wait may suspend the thread for a while first).
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// Arrive where `pred` holds, without a branch.
+__device__ __forceinline__ void mbar_arrive_if(uint64_t* bar, bool pred)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(smem_addr(bar)),
+        "r"((uint32_t)pred)
+        : "memory");
+}
+
 // Wait for the phase with the given parity to complete; give up after
 // kSpinLimit polls, record kErrTimeout in *err and return false.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int32_t* err)
 {
     for (uint32_t i = 0; i < kSpinLimit; ++i)
         if (mbar_try_wait(bar, parity)) return true;
+    atomicExch(err, kErrTimeout);
+    return false;
+}
+
+// mbar_wait without suspending the thread between polls: for waits of a few
+// hundred cycles on the same CTA's warps.
+__device__ __forceinline__ bool mbar_spin(uint64_t* bar, uint32_t parity, int32_t* err)
+{
+    for (uint32_t i = 0; i < kSpinLimit; ++i)
+        if (mbar_test(bar, parity)) return true;
     atomicExch(err, kErrTimeout);
     return false;
 }
