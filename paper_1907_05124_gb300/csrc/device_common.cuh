@@ -78,6 +78,39 @@ __device__ __forceinline__ float nmfa_update(float phi, float inv_norm, float xi
     return fmaf(alpha, shat - s_old, s_old);
 }
 
+// Two FP32 operations in one instruction, each rounded as fmaf, __fadd_rn and
+// __fmul_rn round theirs.
+__device__ __forceinline__ unsigned long long pack2(float2 v)
+{
+    unsigned long long x;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(v.x), "f"(v.y));
+    return x;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long x)
+{
+    float2 v;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(x));
+    return v;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
+    return unpack2(d);
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(d);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(d);
+}
+
 template <typename T>
 __device__ __forceinline__ T shfl_xor(T v, int mask)
 {

@@ -22,6 +22,31 @@ namespace {
 
 constexpr int kWideThreads = 1024;
 
+// One coupling: (column, weight). Format 0: (column, float bits) pairs;
+// format 1: +-1 words, column | sign << 31.
+template <int FMT>
+struct Entry;
+template <>
+struct Entry<1> {
+    const uint32_t* e;
+    __device__ void get(int idx, int& col, float& w) const
+    {
+        const uint32_t v = __ldg(e + idx);
+        col = (int)(v & 0x7fffffffu);
+        w = (v >> 31) ? -1.f : 1.f;
+    }
+};
+template <>
+struct Entry<0> {
+    const int2* e;
+    __device__ void get(int idx, int& col, float& w) const
+    {
+        const int2 v = __ldg(e + idx);
+        col = v.x;
+        w = __int_as_float(v.y);
+    }
+};
+
 // Start states and per-slot schedule state. Grid-stride over
 // groups x (n+1) x RT magnetisations; the first `slots` threads also set up
 // their slot's level.

@@ -677,7 +677,8 @@ int mars_instance_csr(mars_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
     std::vector<int32_t> lvl_slice(nlev + 1, 0);
     std::vector<int32_t> slice_words;  // row0, rows, degree, offset per slice
     std::vector<uint32_t> sell_pm1;
-    std::vector<uint16_t> sell16;      // the same as halfwords when every column fits 15 bits
+    std::vector<uint32_t> sell16;      // two +-1 couplings per word when every column fits 15 bits
+    int32_t odd = 0;                   // slices of odd degree so far (their last word is half padding)
     const bool half = pm1 && n < 32768;
     std::vector<int32_t> sell_gen;     // (column, float bits) pairs
     int64_t sell_len = 0;
@@ -686,18 +687,21 @@ int mars_instance_csr(mars_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
             const int32_t rows = std::min(32, lvl_start[l + 1] - r0);
             int32_t deg = 0;
             for (int32_t q = 0; q < rows; ++q) deg = std::max(deg, nrp[r0 + q + 1] - nrp[r0 + q]);
-            slice_words.insert(slice_words.end(), {r0, rows, deg, (int32_t)sell_len});
+            slice_words.insert(slice_words.end(), {r0, rows, half ? deg | odd << 16 : deg, (int32_t)sell_len});
+            auto entry = [&](int32_t t, int32_t q, double* w) {  // coupling t of row q, or padding
+                if (q >= rows || t >= nrp[r0 + q + 1] - nrp[r0 + q]) {
+                    *w = 0.0;
+                    return n;
+                }
+                *w = nval_f64[nrp[r0 + q] + t];
+                return ncol[nrp[r0 + q] + t];
+            };
             for (int32_t t = 0; t < deg; ++t) {
                 for (int32_t q = 0; q < 32; ++q) {
-                    int32_t cidx = n;
-                    double w = 0.0;
-                    if (q < rows && t < nrp[r0 + q + 1] - nrp[r0 + q]) {
-                        cidx = ncol[nrp[r0 + q] + t];
-                        w = nval_f64[nrp[r0 + q] + t];
-                    }
+                    double w;
+                    const int32_t cidx = entry(t, q, &w);
                     if (pm1) {
                         sell_pm1.push_back((uint32_t)cidx | (w < 0 ? 0x80000000u : 0u));
-                        if (half) sell16.push_back((uint16_t)((uint32_t)cidx | (w < 0 ? 0x8000u : 0u)));
                     } else {
                         const float wf = (float)w;
                         int32_t bits;
@@ -707,6 +711,17 @@ int mars_instance_csr(mars_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
                     }
                 }
             }
+            for (int32_t t = 0; half && t < deg; t += 2)
+                for (int32_t q = 0; q < 32; ++q) {
+                    uint32_t word = 0;
+                    for (int32_t u = 0; u < 2; ++u) {
+                        double w;
+                        const uint32_t cidx = (uint32_t)entry(t + u, q, &w);
+                        word |= (cidx | (w < 0 ? 0x8000u : 0u)) << (16 * u);
+                    }
+                    sell16.push_back(word);
+                }
+            odd += half ? deg & 1 : 0;
             sell_len += (int64_t)deg * 32;
             if (sell_len > INT32_MAX) return fail(c, MARS_EINVAL, "padded coupling table too large");
         }
@@ -728,7 +743,9 @@ int mars_instance_csr(mars_ctx* c, int32_t n, int64_t nnz, const int32_t* row_pt
         if ((rc = upload(c, in.get(), sell_pm1, &d.sell_pm1))) return rc;
         if ((rc = upload(c, in.get(), sell16, &d.sell16))) return rc;
         d.nslices = (int32_t)(slice_words.size() / 4);
+        for (int32_t l = 0; l < nlev; ++l) d.max_slices = std::max(d.max_slices, lvl_slice[l + 1] - lvl_slice[l]);
         d.sell_len = sell_len;
+        d.sell16_len = (int64_t)sell16.size();
         int32_t deg0 = rp[1] - rp[0];
         for (int32_t i = 1; i < n && deg0 >= 0; ++i)
             if (rp[i + 1] - rp[i] != deg0) deg0 = -1;
@@ -1140,8 +1157,9 @@ int mars_solve_batch(mars_ctx* c, int32_t count, const int32_t* insts, const mar
         s.rt = 1;
     }
     BatchPlan bp;
-    std::vector<int> fmts(count), rts(count);
-    if (!plan_sparse_batch(dins.data(), count, c->device, &bp, fmts.data(), rts.data()))
+    std::vector<int> fmts(count), rts(count), nrep(count);
+    for (int32_t j = 0; j < count; ++j) nrep[j] = params[j].replicas;
+    if (!plan_sparse_batch(dins.data(), nrep.data(), count, c->device, &bp, fmts.data(), rts.data()))
         return fail(c, MARS_EINVAL, "an instance is too large for the batched on-chip kernel");
     for (int32_t j = 0; j < count; ++j) {
         jobs[j].fmt = fmts[j];
@@ -1151,7 +1169,19 @@ int mars_solve_batch(mars_ctx* c, int32_t count, const int32_t* insts, const mar
     int32_t* cursor = nullptr;
     if ((rc = S.get(count, &djobs))) return rc;
     if ((rc = S.get(1, &cursor))) return rc;
-    MARS_CUDA(c, cudaMemcpyAsync(djobs, jobs.data(), count * sizeof(BatchJob), cudaMemcpyHostToDevice, st));
+    // The CTAs take the jobs in order: those whose longest replica takes
+    // longest first (temperature levels x colour levels x the work of a row).
+    std::vector<double> length(count);
+    std::vector<int32_t> turn(count);
+    for (int32_t j = 0; j < count; ++j) {
+        const DevInstance& d = dins[j];
+        length[j] = std::max(levels_bound(&params[j], params[j].t_max), 0.0) * d.nlev * (8.0 + (double)d.nnz / d.n);
+    }
+    std::iota(turn.begin(), turn.end(), 0);
+    std::stable_sort(turn.begin(), turn.end(), [&](int32_t a, int32_t b) { return length[a] > length[b]; });
+    std::vector<BatchJob> in_turn(count);
+    for (int32_t q = 0; q < count; ++q) in_turn[q] = jobs[turn[q]];
+    MARS_CUDA(c, cudaMemcpyAsync(djobs, in_turn.data(), count * sizeof(BatchJob), cudaMemcpyHostToDevice, st));
     MARS_CUDA(c, cudaMemsetAsync(cursor, 0, sizeof(int32_t), st));
     MARS_CUDA(c, cudaEventRecord(c->ev0, st));
     MARS_CUDA(c, launch_sparse_batch(djobs, count, cursor, bp, st));

@@ -41,8 +41,14 @@ struct DevInstance {
     const int32_t* lvl_slice = nullptr;  // nlev+1 offsets into slices
     const uint32_t* sell_pm1 = nullptr;  // +-1 couplings: column | sign << 31
     const int2* sell_gen = nullptr;      // general couplings: (column, float bits)
-    const uint16_t* sell16 = nullptr;    // +-1 couplings, n < 32768: column | sign << 15
+    // +-1 couplings, n < 32768: two halfwords (column | sign << 15) per word,
+    // 32 words per pair of couplings of a slice. Its slices then hold their
+    // degree in the low half of .z and the odd-degree slices before them in
+    // the high half: a slice's words start at (.w + 32 odd) / 2.
+    const uint32_t* sell16 = nullptr;
+    int64_t sell16_len = 0;              // words
     int32_t nslices = 0;
+    int32_t max_slices = 0;              // most slices of one level
     int64_t sell_len = 0;                // padded entries (32 x degree summed over slices)
     int32_t regular_deg = 0;             // the common degree when every spin has the same, else 0
     // dense (n*n, new labels: Jn[a][b] = J[new2old[a]][new2old[b]])
@@ -177,7 +183,8 @@ struct BatchPlan {
     size_t smem = 0;
     int grid = 0;
 };
-bool plan_sparse_batch(const DevInstance* ins, int count, int device, BatchPlan* p, int* fmts, int* rts);
+bool plan_sparse_batch(const DevInstance* ins, const int* reps, int count, int device, BatchPlan* p, int* fmts,
+                       int* rts);
 cudaError_t launch_sparse_batch(const BatchJob* jobs, int count, int* cursor, const BatchPlan& p,
                                 cudaStream_t st);
 

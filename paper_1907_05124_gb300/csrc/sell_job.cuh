@@ -12,6 +12,9 @@
 #include "schedule.cuh"
 #include "mars_internal.h"
 
+#include <climits>
+#include <cstdlib>
+
 namespace mars {
 namespace {
 
@@ -66,53 +69,247 @@ struct Vec<4> {
     }
 };
 
-// One coupling: (column, weight). Format 0: (column, float bits) pairs;
-// format 1: +-1 words, column | sign << 31; format 2: +-1 halfwords,
-// column | sign << 15, staged in shared memory for the whole kernel;
-// format 3: the same halfwords read from global memory through L1.
+// Coupling formats. 0: (column, float bits) pairs; 1: +-1 words, column |
+// sign << 31; 2: +-1 halfwords, column | sign << 15, two to a word, staged in
+// shared memory for the whole kernel; 3: the same words read from global
+// memory through L1. A slice's entries are slot-major (DevInstance): entry d of
+// a lane's row is 32 d further on, in formats 2 and 3 a pair of entries.
 template <int FMT>
-struct Entry;
+struct Couplings;
 template <>
-struct Entry<1> {
-    const uint32_t* e;
-    __device__ void get(int idx, int& col, float& w) const
-    {
-        const uint32_t v = __ldg(e + idx);
-        col = (int)(v & 0x7fffffffu);
-        w = (v >> 31) ? -1.f : 1.f;
-    }
-};
-template <>
-struct Entry<0> {
+struct Couplings<0> {
     const int2* e;
-    __device__ void get(int idx, int& col, float& w) const
-    {
-        const int2 v = __ldg(e + idx);
-        col = v.x;
-        w = __int_as_float(v.y);
-    }
 };
 template <>
-struct Entry<2> {
-    const uint16_t* e;  // shared memory
-    __device__ void get(int idx, int& col, float& w) const
-    {
-        const uint32_t v = e[idx];
-        col = (int)(v & 0x7fffu);
-        w = (v >> 15) ? -1.f : 1.f;
-    }
+struct Couplings<1> {
+    const uint32_t* e;
+};
+template <>
+struct Couplings<2> {
+    const uint32_t* e;  // shared memory
+};
+template <>
+struct Couplings<3> {
+    const uint32_t* e;
 };
 
-template <>
-struct Entry<3> {
-    const uint16_t* e;  // the halfword table in global memory, read through L1
-    __device__ void get(int idx, int& col, float& w) const
-    {
-        const uint32_t v = __ldg(e + idx);
-        col = (int)(v & 0x7fffu);
-        w = (v >> 15) ? -1.f : 1.f;
+// acc += w m for one gathered row of W replicas and w = +-1, the sign of `sg`.
+// The product is exact, so this rounds as an FMA does.
+template <int W>
+__device__ __forceinline__ void add_signed(float (&acc)[W], const float* p, uint32_t sg)
+{
+    if constexpr (W == 1) {
+        acc[0] += __uint_as_float(__float_as_uint(p[0]) ^ (sg & 0x80000000u));
+    } else {
+        const float w = __uint_as_float((sg & 0x80000000u) | 0x3f800000u);
+        const float2 ww = make_float2(w, w);
+#pragma unroll
+        for (int k = 0; k < W; k += 2) {
+            const float2 v = fma2(ww, make_float2(p[k], p[k + 1]), make_float2(acc[k], acc[k + 1]));
+            acc[k] = v.x;
+            acc[k + 1] = v.y;
+        }
     }
-};
+}
+
+template <int W>
+__device__ __forceinline__ void add_weighted(float (&acc)[W], const float* p, float w)
+{
+#pragma unroll
+    for (int k = 0; k < W; ++k) acc[k] = fmaf(w, p[k], acc[k]);
+}
+
+// The W replicas' magnetisations of row c (W = 1: one slot of a wider tile).
+template <int RT, int W>
+__device__ __forceinline__ void gather(float (&v)[W], const float* m, uint32_t c)
+{
+    if constexpr (W == 1) {
+        v[0] = m[c * RT];
+    } else {
+        const typename Vec<W>::T x = Vec<W>::load(m + c * RT);
+#pragma unroll
+        for (int k = 0; k < W; ++k) v[k] = Vec<W>::get(x, k);
+    }
+}
+
+// NP pairs of +-1 couplings: their words, then every gather, then the sums in
+// the couplings' order, so that one round trip serves them all.
+template <int RT, int W, int NP>
+__device__ __forceinline__ void field_pairs(float (&acc)[W], const uint32_t (&w)[NP], const float* m)
+{
+    float v[2 * NP][W];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        gather<RT, W>(v[2 * p], m, w[p] & 0x7fffu);
+        gather<RT, W>(v[2 * p + 1], m, (w[p] >> 16) & 0x7fffu);
+    }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        add_signed<W>(acc, v[2 * p], w[p] << 16);
+        add_signed<W>(acc, v[2 * p + 1], w[p]);
+    }
+}
+
+// Local fields of one row for W replicas: acc += sum over its couplings, in
+// their order. e0: the lane's first entry; DEG: the degree when it is known.
+template <int RT, int W, int FMT, int DEG>
+__device__ __forceinline__ void row_field(float (&acc)[W], const Couplings<FMT>& ent, int e0, int deg, const float* m)
+{
+    if constexpr (FMT == 2 || FMT == 3) {
+        const uint32_t* e = ent.e + e0;
+        auto word = [&](int p) { return FMT == 2 ? e[32 * p] : __ldg(e + 32 * p); };
+        if constexpr (DEG > 0) {
+            static_assert(DEG % 2 == 0, "pairs");
+            uint32_t w[DEG / 2];
+#pragma unroll
+            for (int p = 0; p < DEG / 2; ++p) w[p] = word(p);
+            field_pairs<RT, W>(acc, w, m);
+        } else {
+            // batches of four pairs, the next batch's words loaded before this
+            // one's gathers are summed; then two pairs, then one
+            constexpr int B = W > 2 ? 2 : 4;
+            const int np = (deg + 1) >> 1;
+            int p = 0;
+            if (np >= B) {
+                uint32_t w[B];
+#pragma unroll
+                for (int q = 0; q < B; ++q) w[q] = word(q);
+                for (p = B; p + B <= np; p += B) {
+                    uint32_t nw[B];
+#pragma unroll
+                    for (int q = 0; q < B; ++q) nw[q] = word(p + q);
+                    field_pairs<RT, W>(acc, w, m);
+#pragma unroll
+                    for (int q = 0; q < B; ++q) w[q] = nw[q];
+                }
+                field_pairs<RT, W>(acc, w, m);
+            }
+            if (B > 2 && p + 2 <= np) {
+                const uint32_t w[2] = {word(p), word(p + 1)};
+                field_pairs<RT, W>(acc, w, m);
+                p += 2;
+            }
+            if (p < np) {
+                const uint32_t w[1] = {word(p)};
+                field_pairs<RT, W>(acc, w, m);
+            }
+        }
+    } else if constexpr (FMT == 1) {
+        const uint32_t* e = ent.e + e0;
+        const int n = DEG > 0 ? DEG : deg;
+#pragma unroll(DEG > 0 ? DEG : 4)
+        for (int q = 0; q < n; ++q) {
+            const uint32_t w = __ldg(e + 32 * q);
+            float v[W];
+            gather<RT, W>(v, m, w & 0x7fffffffu);
+            add_signed<W>(acc, v, w);
+        }
+    } else {
+        const int2* e = ent.e + e0;
+#pragma unroll 4
+        for (int q = 0; q < deg; ++q) {
+            const int2 w = __ldg(e + 32 * q);
+            float v[W];
+            gather<RT, W>(v, m, (uint32_t)w.x);
+            add_weighted<W>(acc, v, __int_as_float(w.y));
+        }
+    }
+}
+
+// -tanh(x) for the negated argument nx = -x (tanh_sfu; both halves of its
+// formula are odd), for W replicas.
+template <int W>
+__device__ __forceinline__ void neg_tanh(float (&sn)[W], const float (&nx)[W])
+{
+    if constexpr (W == 1) {
+        sn[0] = tanh_sfu(nx[0]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < W; k += 2) {
+            float2 e, r;
+            const float a0 = fabsf(nx[k]) * 2.8853900817779268f, a1 = fabsf(nx[k + 1]) * 2.8853900817779268f;
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(a0));
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(a1));
+            e = add2(e, make_float2(1.0f, 1.0f));
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(e.x));
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(e.y));
+            const float2 b = fma2(make_float2(-2.0f, -2.0f), r, make_float2(1.0f, 1.0f));
+            sn[k] = fabsf(nx[k]) < 4e-3f ? nx[k] : copysignf(b.x, nx[k]);
+            sn[k + 1] = fabsf(nx[k + 1]) < 4e-3f ? nx[k + 1] : copysignf(b.y, nx[k + 1]);
+        }
+    }
+}
+
+// One row's update for W replicas (slots k0 .. k0 + W - 1 of the tile when
+// m points at slot k0 of row 0): s_i <- -tanh(Phi_i / T), the largest change
+// folded into d.
+template <int RT, int W, int FMT, int DEG>
+__device__ __forceinline__ void update_row(const Couplings<FMT>& ent, int e0, int deg, float* m, int i, const float* h,
+                                           const float (&ninvT)[W], float (&d)[W])
+{
+    float acc[W], old[W], nx[W], sn[W];
+#pragma unroll
+    for (int k = 0; k < W; ++k) acc[k] = 0.f;
+    gather<RT, W>(old, m, (uint32_t)i);
+    row_field<RT, W, FMT, DEG>(acc, ent, e0, deg, m);
+    if (h) {
+        const float hv = __ldg(h + i);
+#pragma unroll
+        for (int k = 0; k < W; ++k) acc[k] += hv;
+    }
+#pragma unroll
+    for (int k = 0; k < W; ++k) nx[k] = acc[k] * ninvT[k];
+    neg_tanh<W>(sn, nx);
+#pragma unroll
+    for (int k = 0; k < W; ++k) d[k] = fmaxf(d[k], fabsf(sn[k] - old[k]));
+    if constexpr (W == 1) {
+        m[i * RT] = sn[0];
+    } else {
+        typename Vec<W>::T v;
+#pragma unroll
+        for (int k = 0; k < W; ++k) Vec<W>::set(v, k, sn[k]);
+        Vec<W>::store(m + i * RT, v);
+    }
+}
+
+// The levels of one sweep in order, each a parallel step over the CTA's warps
+// (32-row slices), with a barrier after all but the last.
+template <int RT, int W, int NT, int FMT, int DEG>
+__device__ __forceinline__ void sweep_levels(const DevInstance& in, const Couplings<FMT>& ent, const int4* slices,
+                                             float* m, const float (&ninvT)[W], float (&d)[W])
+{
+    constexpr int kWarps = NT / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int s0 = 0, s1 = __ldg(in.lvl_slice + 1);  // this level's slices; level 0 starts at 0
+    int r0 = 0, r1 = DEG > 0 ? __ldg(in.lvl_start + 1) : 0;
+    for (int l = 0; l < in.nlev; ++l) {
+        // the next level's bounds arrive while this one runs
+        const int ln = l + 2 <= in.nlev ? l + 2 : in.nlev;
+        const int s2 = __ldg(in.lvl_slice + ln);
+        const int r2 = DEG > 0 ? __ldg(in.lvl_start + ln) : 0;
+        if constexpr (DEG > 0) {
+            // every slice has degree DEG: its rows and couplings follow from its number
+            constexpr int kE = FMT >= 2 ? 16 * DEG : 32 * DEG;
+            int i = r0 + 32 * warp + lane;
+            for (int sl = s0 + warp; sl < s1; sl += kWarps, i += 32 * kWarps)
+                if (i < r1) update_row<RT, W, FMT, DEG>(ent, sl * kE + lane, DEG, m, i, in.h, ninvT, d);
+        } else {
+            for (int sl = s0 + warp; sl < s1; sl += kWarps) {
+                const int4 c = FMT == 2 ? slices[sl] : __ldg(slices + sl);  // row0, rows, degree, offset
+                if (lane >= c.y) continue;
+                const bool half = FMT >= 2 || (FMT == 1 && in.sell16);  // .z holds two numbers
+                const int deg = half ? c.z & 0xffff : c.z;
+                const int e0 = FMT >= 2 ? ((c.w + 32 * (int)((uint32_t)c.z >> 16)) >> 1) + lane : c.w + lane;
+                update_row<RT, W, FMT, 0>(ent, e0, deg, m, c.x + lane, in.h, ninvT, d);
+            }
+        }
+        if (l + 1 < in.nlev) __syncthreads();
+        s0 = s1;
+        s1 = s2;
+        r0 = r1;
+        r1 = r2;
+    }
+}
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
@@ -124,6 +321,24 @@ __host__ __device__ inline size_t sell_slab_floats(int n, int rt)
     return align16((size_t)(n + 1) * rt * sizeof(float)) / sizeof(float);
 }
 
+// Bytes of the slice table and the +-1 halfword couplings (format 2).
+inline size_t half_table_bytes(const DevInstance& in)
+{
+    return (size_t)in.nslices * sizeof(int4) + (size_t)in.sell16_len * sizeof(uint32_t);
+}
+
+// Whether a solve of R replicas takes one slot per CTA (plan_sparse_sell).
+inline bool few_replicas(const DevInstance& in, int R, int sms)
+{
+    return R <= 2 * sms || (2 * R <= 7 * sms && in.nnz <= (int64_t)16 * in.n);
+}
+
+inline int env_int(const char* name, int dflt)
+{
+    const char* v = std::getenv(name);
+    return v && *v ? std::atoi(v) : dflt;
+}
+
 // Per-CTA bookkeeping of the RT replica slots, in shared memory.
 template <int RT, int NW>
 struct SlotState {
@@ -131,7 +346,7 @@ struct SlotState {
     float invT[RT];
     int rep[RT], fresh[RT], done[RT];
     int lvl_sweeps[RT], sweeps[RT], levels[RT], capped[RT], active[RT];
-    float dred[NW][RT];
+    uint32_t dred[2][NW][RT];  // per-warp largest changes (float bits), by sweep parity
     long long ei[NW][RT];
     double ef[NW][RT];
 };
@@ -163,19 +378,19 @@ __device__ void run_job(const DevInstance& in, const DevSolve& s, float* m, Slot
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = in.n;
     __shared__ int s_last[RT];  // serving ring: this slot finished its job's last replica
-    Entry<FMT> ent;
+    Couplings<FMT> ent;
     const int4* slices = in.slices;
     if constexpr (FMT == 0) ent.e = in.sell_gen;
     if constexpr (FMT == 1) ent.e = in.sell_pm1;
     if constexpr (FMT == 3) ent.e = in.sell16;
     if constexpr (FMT == 2) {
-        // Stage the slice table and the halfword couplings in shared memory,
-        // after the magnetisations; they serve every replica this CTA runs.
+        // Stage the slice table and the couplings in shared memory, after the
+        // magnetisations; they serve every replica this CTA runs.
         unsigned char* base = reinterpret_cast<unsigned char*>(m);
         int4* ss = reinterpret_cast<int4*>(base + align16((size_t)(n + 1) * RT * sizeof(float)));
-        uint16_t* se = reinterpret_cast<uint16_t*>(ss + in.nslices);
+        uint32_t* se = reinterpret_cast<uint32_t*>(ss + in.nslices);
         for (int q = tid; q < in.nslices; q += kThreads) ss[q] = __ldg(in.slices + q);
-        for (int64_t q = tid; q < in.sell_len; q += kThreads) se[q] = __ldg(in.sell16 + q);
+        for (int64_t q = tid; q < in.sell16_len; q += kThreads) se[q] = __ldg(in.sell16 + q);
         slices = ss;
         ent.e = se;
         __syncthreads();
@@ -343,127 +558,84 @@ __device__ void run_job(const DevInstance& in, const DevSolve& s, float* m, Slot
         for (int k = 0; k < RT; ++k) { act[k] = s_active[k] != 0; any_act |= act[k]; }
         if (!any_act) break;  // every slot is empty: the queue ran dry
 
-        // ---- one sweep: the levels in order, each a parallel step -------------
+        // ---- sweeps until a slot's level ends --------------------------------
         // A thread updates its spin for all RT replicas from one coupling load
-        // and RT-wide gathers (dead slots skip only their tanh). When a single
-        // slot is left (the queue ran dry) it takes a one-replica path, so a
-        // straggler replica's sweep costs what a one-replica sweep costs.
-        float invT[RT], dloc[RT];
-        int live = 0;
+        // and RT-wide gathers (a dead slot's values are computed and never
+        // used). When a single slot is left (the queue ran dry) it takes a
+        // one-replica path, so a straggler's sweep costs what a one-replica
+        // sweep costs. Every thread applies the stopping rule to every slot
+        // itself, from the warps' largest changes: a sweep has one barrier per
+        // level and no other.
+        int live = 0, only = 0;
+        float ninvT[RT], dmin[RT];
+        int ls[RT], limit[RT], done_now[RT];
 #pragma unroll
         for (int k = 0; k < RT; ++k) {
-            invT[k] = s_invT[k];
-            dloc[k] = 0.f;
-            live |= act[k] ? 1 << k : 0;
+            ninvT[k] = act[k] ? -s_invT[k] : 0.f;
+            live += act[k];
+            only = act[k] ? k : only;
+            const bool fixed = sched_fixed(s, s_T[k]);
+            ls[k] = act[k] ? s_lvl_sweeps[k] : 0;
+            limit[k] = act[k] ? (fixed ? s.fixed_sweeps : s.k_max) : INT_MAX;
+            dmin[k] = act[k] && !fixed ? s.d_min : -1.f;  // changes are >= 0
+            done_now[k] = 0;
         }
-        const bool all_live = RT == 1 || __popc(live) > 1;
-        const bool lean = live == (1 << RT) - 1 && !in.h;  // uniform over the CTA
-        for (int l = 0; l < in.nlev; ++l) {
-            const int s0 = __ldg(in.lvl_slice + l), s1 = __ldg(in.lvl_slice + l + 1);
-            for (int sl = s0 + warp; sl < s1; sl += kWarps) {
-                const int4 d = FMT == 2 ? slices[sl] : __ldg(in.slices + sl);  // row0, rows, degree, offset
-                if (lane >= d.y) continue;
-                const int i = d.x + lane;
-                const float hv = in.h ? __ldg(in.h + i) : 0.f;
-                if (all_live) {
-                    typename V::T acc;
+        int sweeps = 0, par = 0;
+        float dd[RT];
+        for (bool more = true; more; par ^= 1) {
+            float d[RT];
 #pragma unroll
-                    for (int k = 0; k < RT; ++k) V::set(acc, k, 0.f);
-                    const int deg = DEG > 0 ? DEG : d.z;  // a regular instance's degree is known
-#pragma unroll 4
-                    for (int q = 0; q < deg; ++q) {
-                        int c;
-                        float w;
-                        ent.get(d.w + 32 * q + lane, c, w);
-                        const typename V::T mv = V::load(m + c * RT);
+            for (int k = 0; k < RT; ++k) d[k] = 0.f;
+            if (RT > 1 && live == 1) {
+                float d1[1] = {0.f}, n1[1] = {ninvT[0]};
 #pragma unroll
-                        for (int k = 0; k < RT; ++k)
-                            V::set(acc, k, fmaf(w, V::get(mv, k), V::get(acc, k)));
-                    }
-                    const typename V::T old = V::load(m + i * RT);
-                    typename V::T nv;
-                    if (lean) {
-                        // every slot live, no field: no per-slot test, no add
+                for (int k = 1; k < RT; ++k)
+                    if (only == k) n1[0] = ninvT[k];
+                sweep_levels<RT, 1, NT, FMT, DEG>(in, ent, slices, m + only, n1, d1);
 #pragma unroll
-                        for (int k = 0; k < RT; ++k) {
-                            const float sn = -tanh_sfu(V::get(acc, k) * invT[k]);
-                            dloc[k] = fmaxf(dloc[k], fabsf(sn - V::get(old, k)));
-                            V::set(nv, k, sn);
-                        }
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < RT; ++k) {
-                            if ((live >> k) & 1) {
-                                const float sn = -tanh_sfu((V::get(acc, k) + hv) * invT[k]);
-                                dloc[k] = fmaxf(dloc[k], fabsf(sn - V::get(old, k)));
-                                V::set(nv, k, sn);
-                            } else {
-                                V::set(nv, k, V::get(old, k));
-                            }
-                        }
-                    }
-                    V::store(m + i * RT, nv);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < RT; ++k) {
-                        if (!((live >> k) & 1)) continue;
-                        float acc = 0.f;
-                        const int deg = DEG > 0 ? DEG : d.z;
-#pragma unroll 4
-                        for (int q = 0; q < deg; ++q) {
-                            int c;
-                            float w;
-                            ent.get(d.w + 32 * q + lane, c, w);
-                            acc = fmaf(w, m[c * RT + k], acc);
-                        }
-                        const float old = m[i * RT + k];
-                        const float sn = -tanh_sfu((acc + hv) * invT[k]);
-                        dloc[k] = fmaxf(dloc[k], fabsf(sn - old));
-                        m[i * RT + k] = sn;
-                    }
-                }
+                for (int k = 0; k < RT; ++k)
+                    if (only == k) d[k] = d1[0];
+            } else {
+                sweep_levels<RT, RT, NT, FMT, DEG>(in, ent, slices, m, ninvT, d);
             }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int k = 0; k < RT; ++k) {
-            const float v = warp_reduce_strided<1>(dloc[k], MaxOp());
-            if (lane == 0) s_dred[warp][k] = v;
-        }
-        __syncthreads();
-        if (warp == 0) {
-            // the per-warp maxima of each slot, reduced by warp 0's lanes
-            float dk[RT];
 #pragma unroll
             for (int k = 0; k < RT; ++k) {
-                float v = lane < kWarps ? s_dred[lane][k] : 0.f;
-                dk[k] = warp_reduce_strided<1>(v, MaxOp());
+                // non-negative floats order like their bits
+                const uint32_t v = __reduce_max_sync(0xffffffffu, __float_as_uint(d[k]));
+                if (lane == 0) s_dred[par][warp][k] = v;
             }
-            if (lane < RT && s_active[lane]) {
-                const int k = lane;
-                float dd = dk[0];
+            __syncthreads();  // the last level's spins and the warps' changes
+            ++sweeps;
 #pragma unroll
-                for (int q = 1; q < RT; ++q)
-                    if (q == k) dd = dk[q];
-                int ls = s_lvl_sweeps[k] + 1;
-                s_sweeps[k] += 1;
-                double T = s_T[k];
-                const bool fixed = sched_fixed(s, T);
-                const bool level_done = fixed ? ls >= s.fixed_sweeps : (dd <= s.d_min || ls >= s.k_max);
-                if (level_done) {
-                    if (!fixed && !(dd <= s.d_min)) s_capped[k] += 1;
-                    ls = 0;
-                    if (sched_advance(s, &T)) {
-                        s_T[k] = T;
-                        s_levels[k] += 1;
-                        s_invT[k] = sched_inv_t(T);
-                    } else {
-                        s_active[k] = 0;
-                        s_done[k] = 1;
-                    }
-                }
-                s_lvl_sweeps[k] = ls;
+            for (int k = 0; k < RT; ++k) {
+                const uint32_t v = lane < kWarps ? s_dred[par][lane][k] : 0u;
+                dd[k] = __uint_as_float(__reduce_max_sync(0xffffffffu, v));
+                ls[k] += 1;
+                done_now[k] = dd[k] <= dmin[k] || ls[k] >= limit[k];
+                more &= !done_now[k];
             }
+        }
+        // the levels that ended: cool, or finish (the slots' sweeps so far)
+        __syncthreads();  // every thread has read the slots' state
+#pragma unroll
+        for (int k = 0; k < RT; ++k) {
+            if (tid != k || !act[k]) continue;
+            s_sweeps[k] += sweeps;
+            double T = s_T[k];
+            int l = ls[k];
+            if (done_now[k]) {
+                if (!sched_fixed(s, T) && !(dd[k] <= s.d_min)) s_capped[k] += 1;
+                l = 0;
+                if (sched_advance(s, &T)) {
+                    s_T[k] = T;
+                    s_levels[k] += 1;
+                    s_invT[k] = sched_inv_t(T);
+                } else {
+                    s_active[k] = 0;
+                    s_done[k] = 1;
+                }
+            }
+            s_lvl_sweeps[k] = l;
         }
         __syncthreads();
     }
