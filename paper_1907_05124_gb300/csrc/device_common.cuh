@@ -111,6 +111,13 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b)
     return unpack2(d);
 }
 
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    unsigned long long d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(d);
+}
+
 template <typename T>
 __device__ __forceinline__ T shfl_xor(T v, int mask)
 {
