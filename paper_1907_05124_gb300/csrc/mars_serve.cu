@@ -42,6 +42,7 @@ struct ServeReq {
     DevResult* dres = nullptr;
     int8_t* dbest = nullptr;
     unsigned char* pinned = nullptr;  // DevResult | status | counters[4] | best spins
+    size_t pinned_bytes = 0;
     cudaEvent_t ev = nullptr;
     std::unique_ptr<TcRun> tc;
     double total_weight = 0.0, err_bound = 0.0;
@@ -87,7 +88,41 @@ struct Serve {
     // the device is left to the dense requests' kernels.
     int sparse_sms = 0;
     int sms = 0;
+    // Result blocks of collected requests, for the next ones: allocating and
+    // freeing pinned memory waits for the whole device, so a submit or poll
+    // that did either stood still until the serving kernel and every other
+    // request had ended. At most kPinnedKeep bytes are kept, and the engine
+    // frees them with itself.
+    std::multimap<size_t, unsigned char*> pinned_free;
+    size_t pinned_kept = 0;
 };
+constexpr size_t kPinnedKeep = (size_t)16 << 20;
+
+// A pinned block of at least `bytes`: a kept one of at most four times the size
+// (or 64 kB), else a new one.
+cudaError_t pinned_get(Serve* sv, size_t bytes, unsigned char** out, size_t* got)
+{
+    auto it = sv->pinned_free.lower_bound(bytes);
+    if (it != sv->pinned_free.end() && it->first <= std::max<size_t>(4 * bytes, 65536)) {
+        *out = it->second;
+        *got = it->first;
+        sv->pinned_kept -= it->first;
+        sv->pinned_free.erase(it);
+        return cudaSuccess;
+    }
+    *got = (bytes + 4095) & ~(size_t)4095;
+    return cudaMallocHost((void**)out, *got);
+}
+
+void pinned_put(Serve* sv, unsigned char* p, size_t bytes)
+{
+    if (sv->pinned_kept + bytes > kPinnedKeep) {
+        cudaFreeHost(p);
+        return;
+    }
+    sv->pinned_free.emplace(bytes, p);
+    sv->pinned_kept += bytes;
+}
 
 // The grid of a persistent sparse launch planned for the whole device, cut to
 // the serving engine's share of the SMs.
@@ -227,7 +262,11 @@ void serve_free_req(mars_ctx* c, Serve* sv, ServeReq* q)
         q->bufs.clear();
     }
     if (q->pinned) {
-        cudaFreeHost(q->pinned);
+        // a failed request may still have copies into the block under way
+        if (q->state == ReqState::Failed && q->st && cudaStreamQuery(q->st) != cudaSuccess)
+            cudaFreeHost(q->pinned);
+        else
+            pinned_put(sv, q->pinned, q->pinned_bytes);
         q->pinned = nullptr;
     }
     if (q->ev) {
@@ -335,7 +374,7 @@ int serve_launch(mars_ctx* c, Serve* sv, ServeReq* q)
         return MARS_OK;
     };
     MARS_CUDA(c, cudaEventCreateWithFlags(&q->ev, cudaEventDisableTiming));
-    MARS_CUDA(c, cudaMallocHost((void**)&q->pinned, 256 + (size_t)n));
+    MARS_CUDA(c, pinned_get(sv, 256 + (size_t)n, &q->pinned, &q->pinned_bytes));
     DevSolve& s = q->s;
     s.R = R;
     s.seed = p.seed;
@@ -618,6 +657,8 @@ void serve_release(mars_ctx* c)
     for (cudaStream_t st : sv->streams) cudaStreamSynchronize(st);
     for (auto& kv : sv->reqs) serve_free_req(c, sv, kv.second.get());
     sv->reqs.clear();
+    for (auto& kv : sv->pinned_free) cudaFreeHost(kv.second);
+    sv->pinned_free.clear();
     for (cudaStream_t st : sv->streams) cudaStreamDestroy(st);
     sv->streams.clear();
     c->serve.reset();
