@@ -678,6 +678,8 @@ __device__ __forceinline__ void advance_slot(const TcState& t, int slot)
 
 __global__ void tc_advance_kernel(TcState t)
 {
+    tc::pdl_wait();  // the sweep's last chain
+    tc::pdl_launch_dependents();
     for (int slot = blockIdx.x * blockDim.x + threadIdx.x; slot < t.R; slot += gridDim.x * blockDim.x)
         advance_slot(t, slot);
 }
@@ -895,6 +897,8 @@ __global__ void tc_prefix_kernel(TcState t)
     __shared__ int s_max, s_cnt;
     if (threadIdx.x == 0) { s_max = 0; s_cnt = 0; }
     __syncthreads();
+    tc::pdl_wait();  // the level step
+    tc::pdl_launch_dependents();
     int mx = 0, cnt = 0;
     for (int slot = threadIdx.x; slot < t.R; slot += blockDim.x)
         if (t.active[slot]) { mx = max(mx, slot + 1); ++cnt; }
@@ -1200,11 +1204,12 @@ cudaError_t launch_tc_sweeps(const CUtensorMap& tmJ, const CUtensorMap& tmS, con
 
 cudaError_t launch_tc_advance(const TcState& t, cudaStream_t st)
 {
-    tc_advance_kernel<<<(t.R + 255) / 256, 256, 0, st>>>(t);
-    cudaError_t e = cudaGetLastError();
+    // programmatic launches, like the sweep's other kernels: each waits itself
+    TcState a = t;
+    void* args[] = {&a};
+    cudaError_t e = launch_pdl((const void*)tc_advance_kernel, dim3((t.R + 255) / 256), dim3(256), args, 0, st);
     if (e != cudaSuccess) return e;
-    tc_prefix_kernel<<<1, 1024, 0, st>>>(t);
-    return cudaGetLastError();
+    return launch_pdl((const void*)tc_prefix_kernel, dim3(1), dim3(1024), args, 0, st);
 }
 
 cudaError_t launch_tc_compact(const TcState& t, int32_t* rep, const TcCompact& cp, int prefix, cudaStream_t st)

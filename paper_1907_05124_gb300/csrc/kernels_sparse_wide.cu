@@ -14,6 +14,7 @@
 // coupling order and passed through the same tanh as in the per-CTA kernels,
 // so a replica's trajectory does not depend on which kernel ran it.
 #include "sell_job.cuh"
+#include "tc_primitives.cuh"
 
 #include <cstdlib>
 
@@ -111,11 +112,12 @@ __global__ void __launch_bounds__(kWideThreads, 1) wide_level_kernel(DevInstance
     (void)s;
     using V = Vec<RT>;
     constexpr int kWarps = kWideThreads / 32;
-    const int ng = w.counters[0];
-    if (ng == 0) return;
     const int s0 = __ldg(in.lvl_slice + l), s1 = __ldg(in.lvl_slice + l + 1);
     const int nsl = s1 - s0;
-    if (nsl <= 0) return;
+    tc::pdl_wait();  // the level, or the decision, before this one
+    tc::pdl_launch_dependents();
+    const int ng = w.counters[0];
+    if (ng == 0 || nsl <= 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     Entry<FMT> ent;
     if constexpr (FMT == 0) ent.e = in.sell_gen;
@@ -147,7 +149,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) wide_level_kernel(DevInstance
         if (it < b1) {
             const int gi = (int)(it / nsl);
             sl = (int)(it - (int64_t)gi * nsl);
-            g = __ldg(w.glist + gi);
+            g = w.glist[gi];
 #pragma unroll
             for (int q = 0; q < DEG; ++q) cw[q] = __ldg(ew + (size_t)sl * 32 * DEG + 32 * q);
         }
@@ -158,7 +160,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) wide_level_kernel(DevInstance
             if (itn < b1) {
                 const int gi = (int)(itn / nsl);
                 sln = (int)(itn - (int64_t)gi * nsl);
-                gn = __ldg(w.glist + gi);
+                gn = w.glist[gi];
 #pragma unroll
                 for (int q = 0; q < DEG; ++q) cn[q] = __ldg(ew + (size_t)sln * 32 * DEG + 32 * q);
             } else {
@@ -226,7 +228,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) wide_level_kernel(DevInstance
     for (int64_t it = b0 + warp; it < b1; it += kWarps) {
         const int gi = (int)(it / nsl);
         const int sl = s0 + (int)(it - (int64_t)gi * nsl);
-        const int g = __ldg(w.glist + gi);
+        const int g = w.glist[gi];
         if (g != cur) {
             if (cur >= 0) flush_d<RT>(w, cur, live, dloc, lane);
             cur = g;
@@ -302,7 +304,9 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 // The level kernel for regular +-1 lattices with the neighbour gathers staged
-// in shared memory: while a warp computes item j from its stage, the
+// in shared memory (75 us a level of the L = 64 lattice with 256 replicas live,
+// 5.4 TB/s of algorithmic traffic on a GB300: DRAM and the L1 bound it; with a
+// few groups left the round trips of its start do): while a warp computes item j from its stage, the
 // asynchronous copies of item j+1's gathers (which hold no registers) and the
 // coupling words of item j+2 are in flight, so each SM keeps about twice the
 // loads of the register-pipelined kernel outstanding. The arithmetic per spin
@@ -316,11 +320,12 @@ __global__ void __launch_bounds__(kWideThreads, 1) wide_level_staged_kernel(DevI
     constexpr int kWarps = kWideThreads / 32;
     constexpr int kStage = DEG * 32 * RT;  // floats of one stage
     extern __shared__ float4 wide_stage_smem[];
-    const int ng = w.counters[0];
-    if (ng == 0) return;
     const int s0 = __ldg(in.lvl_slice + l), s1 = __ldg(in.lvl_slice + l + 1);
     const int nsl = s1 - s0;
-    if (nsl <= 0) return;
+    tc::pdl_wait();  // the level, or the decision, before this one
+    tc::pdl_launch_dependents();
+    const int ng = w.counters[0];
+    if (ng == 0 || nsl <= 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t items = (int64_t)ng * nsl;
     const int64_t per = (items + gridDim.x - 1) / gridDim.x;
@@ -371,7 +376,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) wide_level_staged_kernel(DevI
     {
         const int gi = (int)(itA / nsl);
         slA = (int)(itA - (int64_t)gi * nsl);
-        gA = __ldg(w.glist + gi);
+        gA = w.glist[gi];
     }
     couplings(slA);
     uint32_t signA = issue(gA, 0);
@@ -379,11 +384,11 @@ __global__ void __launch_bounds__(kWideThreads, 1) wide_level_staged_kernel(DevI
     typename V::T oldA = old_of(gA, slA);
     int64_t itB = itA + kWarps;
     bool hasB = itB < b1;
-    int gB = gA, slB = 0;
+    int gB = gA, slB = 0, giB = 0;
     if (hasB) {
-        const int gi = (int)(itB / nsl);
-        slB = (int)(itB - (int64_t)gi * nsl);
-        gB = __ldg(w.glist + gi);
+        giB = (int)(itB / nsl);
+        slB = (int)(itB - (int64_t)giB * nsl);
+        gB = w.glist[giB];
         couplings(slB);
     }
 
@@ -405,9 +410,12 @@ __global__ void __launch_bounds__(kWideThreads, 1) wide_level_staged_kernel(DevI
         const bool hasC = hasB && itC < b1;
         int gC = gB, slC = 0;
         if (hasC) {
-            const int gi = (int)(itC / nsl);
-            slC = (int)(itC - (int64_t)gi * nsl);
-            gC = __ldg(w.glist + gi);
+            slC = slB + kWarps;  // the item kWarps further on
+            while (slC >= nsl) {
+                slC -= nsl;
+                ++giB;
+            }
+            gC = w.glist[giB];
             couplings(slC);
         }
         cp_async_wait<1>();  // item A's copies have landed
@@ -477,83 +485,147 @@ __global__ void __launch_bounds__(kWideThreads, 1) wide_level_staged_kernel(DevI
 // After a sweep (step != 0): each live slot's sweep count, the stopping rule
 // on its largest change d, and the cooling step, as in the per-CTA kernels;
 // then (also with step == 0, after the start) the live groups in ascending
-// order and the live group and replica counts. One CTA.
+// order and the live group and replica counts. One CTA, one thread per slot,
+// kWideThreads slots at a time: it runs between the levels of every sweep, so
+// it is one round trip of loads and two barriers (5.2 us as a launch of its own
+// with a load per decision and a barrier per step of a sum).
 __global__ void __launch_bounds__(kWideThreads) wide_decide_kernel(DevSolve s, DevWide w, int step)
 {
-    __shared__ int s_cnt[kWideThreads];
-    __shared__ int s_warp[kWideThreads / 32];
+    __shared__ int s_groups[kWideThreads / 32], s_reps[kWideThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int slots = w.groups * w.rt;
-    if (step) {
-        for (int q = tid; q < slots; q += kWideThreads) {
-            if (!w.live[q]) continue;
-            const float dd = __uint_as_float(w.dmax[q]);
-            w.dmax[q] = 0u;
-            int ls = w.lvl_sweeps[q] + 1;
-            w.sweeps[q] += 1;
+    tc::pdl_wait();  // the sweep's last level
+    tc::pdl_launch_dependents();
+    int groups_before = 0, reps_before = 0;
+    for (int base = 0; base < slots; base += kWideThreads) {
+        const int q = base + tid;
+        bool live = false;
+        if (q < slots) {
+            const int was = w.live[q], ls0 = w.lvl_sweeps[q], sw = w.sweeps[q];
+            const uint32_t dbits = w.dmax[q];
             double T = w.T[q];
-            const bool fixed = sched_fixed(s, T);
-            const bool level_done = fixed ? ls >= s.fixed_sweeps : (dd <= s.d_min || ls >= s.k_max);
-            if (level_done) {
-                if (!fixed && !(dd <= s.d_min)) w.capped[q] += 1;
-                ls = 0;
-                if (sched_advance(s, &T)) {
-                    w.T[q] = T;
-                    w.levels[q] += 1;
-                    w.invT[q] = sched_inv_t(T);
-                } else {
-                    w.live[q] = 0;
+            live = was != 0;
+            if (step && live) {
+                const float dd = __uint_as_float(dbits);
+                w.dmax[q] = 0u;
+                int ls = ls0 + 1;
+                w.sweeps[q] = sw + 1;
+                const bool fixed = sched_fixed(s, T);
+                const bool level_done = fixed ? ls >= s.fixed_sweeps : (dd <= s.d_min || ls >= s.k_max);
+                if (level_done) {
+                    if (!fixed && !(dd <= s.d_min)) w.capped[q] += 1;
+                    ls = 0;
+                    if (sched_advance(s, &T)) {
+                        w.T[q] = T;
+                        w.levels[q] += 1;
+                        w.invT[q] = sched_inv_t(T);
+                    } else {
+                        w.live[q] = 0;
+                        live = false;
+                    }
                 }
+                w.lvl_sweeps[q] = ls;
             }
-            w.lvl_sweeps[q] = ls;
+        }
+        // a group is w.rt neighbouring lanes (1, 2 or 4): its first lane speaks for it
+        const uint32_t flags = __ballot_sync(0xffffffffu, live);
+        const bool any = lane % w.rt == 0 && ((flags >> lane) & ((1u << w.rt) - 1u)) != 0;
+        const uint32_t heads = __ballot_sync(0xffffffffu, any);
+        if (lane == 0) {
+            s_groups[warp] = __popc(heads);
+            s_reps[warp] = __popc(flags);
         }
         __syncthreads();
-    }
-    // ordered compaction: thread t owns the groups [t*per, (t+1)*per)
-    const int G = w.groups;
-    const int per = (G + kWideThreads - 1) / kWideThreads;
-    const int g0 = tid * per, g1 = min(G, g0 + per);
-    int cnt = 0, reps = 0;
-    for (int g = g0; g < g1; ++g) {
-        int any = 0;
-        for (int k = 0; k < w.rt; ++k) any += w.live[g * w.rt + k] != 0;
-        reps += any;
-        cnt += any > 0;
-    }
-    // exclusive scan of cnt over the block
-    int x = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) s_warp[warp] = x;
-    s_cnt[tid] = reps;
-    __syncthreads();
-    if (warp == 0) {
-        int v = lane < kWideThreads / 32 ? s_warp[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += y;
-        }
-        if (lane < kWideThreads / 32) s_warp[lane] = v;  // inclusive warp totals
-    }
-    __syncthreads();
-    int pos = x - cnt + (warp > 0 ? s_warp[warp - 1] : 0);
-    for (int g = g0; g < g1; ++g) {
-        int any = 0;
-        for (int k = 0; k < w.rt; ++k) any |= w.live[g * w.rt + k];
-        if (any) w.glist[pos++] = g;
-    }
-    // live replicas: a plain block sum
-    for (int o = kWideThreads / 2; o > 0; o >>= 1) {
+        const int gw = s_groups[lane], rw = s_reps[lane];  // 32 warps: one each
+        const int before = __reduce_add_sync(0xffffffffu, lane < warp ? gw : 0);
+        if (any) w.glist[groups_before + before + __popc(heads & ((1u << lane) - 1u))] = q / w.rt;
+        groups_before += __reduce_add_sync(0xffffffffu, gw);
+        reps_before += __reduce_add_sync(0xffffffffu, rw);
         __syncthreads();
-        if (tid < o) s_cnt[tid] += s_cnt[tid + o];
     }
     if (tid == 0) {
-        w.counters[0] = s_warp[kWideThreads / 32 - 1];
-        w.counters[1] = s_cnt[0];
+        w.counters[0] = groups_before;
+        w.counters[1] = reps_before;
+    }
+}
+
+// Repacking of the live replicas into full groups. A level launch moves a live
+// group's rows for all RT slots, so once replicas finish here and there the
+// traffic no longer follows the live ones. The plan (one CTA) keeps as few
+// groups as hold every live replica, the fullest first, and pairs each live slot
+// outside them with a dead one inside; the move exchanges the two slots'
+// magnetisations (a finished replica's are still to be returned), and the swap
+// their state. A replica's arithmetic does not depend on its slot.
+constexpr int kRepackSlots = 16384;  // most slots (their live flags sit in shared memory)
+
+__global__ void __launch_bounds__(kWideThreads) wide_repack_plan_kernel(DevWide w)
+{
+    __shared__ uint8_t s_live[kRepackSlots];
+    const int slots = w.groups * w.rt;
+    for (int q = threadIdx.x; q < slots; q += kWideThreads) s_live[q] = w.live[q] != 0;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    auto count = [&](int g) {
+        int c = 0;
+        for (int k = 0; k < w.rt; ++k) c += s_live[g * w.rt + k] & 1;
+        return c;
+    };
+    int total = 0;
+    for (int g = 0; g < w.groups; ++g) total += count(g);
+    int need = (total + w.rt - 1) / w.rt;
+    for (int c = w.rt; c >= 0 && need > 0; --c)  // bit 1 of a group's first flag: kept
+        for (int g = 0; g < w.groups && need > 0; ++g)
+            if (count(g) == c) {
+                s_live[g * w.rt] |= 2;
+                --need;
+            }
+    int pairs = 0, dst = 0;
+    for (int q = 0; q < slots; ++q) {
+        if (!(s_live[q] & 1) || (s_live[q / w.rt * w.rt] & 2)) continue;
+        while (dst < slots && ((s_live[dst] & 1) || !(s_live[dst / w.rt * w.rt] & 2))) ++dst;
+        if (dst >= slots) break;  // the kept groups hold every live replica: not reached
+        w.pairs[pairs++] = make_int2(dst++, q);
+    }
+    w.counters[2] = pairs;
+}
+
+template <int RT>
+__global__ void wide_repack_move_kernel(int n, DevWide w)
+{
+    const int64_t total = (int64_t)w.counters[2] * n;
+    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
+         idx += (int64_t)gridDim.x * blockDim.x) {
+        const int p = (int)(idx / n), i = (int)(idx - (int64_t)p * n);
+        const int2 pr = w.pairs[p];
+        float* a = w.m + (size_t)(pr.x / RT) * w.slab + (size_t)i * RT + pr.x % RT;
+        float* b = w.m + (size_t)(pr.y / RT) * w.slab + (size_t)i * RT + pr.y % RT;
+        const float x = *a, y = *b;
+        *a = y;
+        *b = x;
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ void swap_slots(T* v, int2 p)
+{
+    const T x = v[p.x];
+    v[p.x] = v[p.y];
+    v[p.y] = x;
+}
+
+__global__ void wide_repack_swap_kernel(DevWide w, int32_t* tile_rep)
+{
+    for (int q = threadIdx.x; q < w.counters[2]; q += blockDim.x) {
+        const int2 p = w.pairs[q];
+        swap_slots(w.T, p);
+        swap_slots(w.invT, p);
+        swap_slots(w.live, p);
+        swap_slots(w.lvl_sweeps, p);
+        swap_slots(w.sweeps, p);
+        swap_slots(w.levels, p);
+        swap_slots(w.capped, p);
+        swap_slots(w.dmax, p);
+        swap_slots(tile_rep, p);
     }
 }
 
@@ -728,7 +800,7 @@ cudaError_t launch_wide_level(const DevInstance& in, const DevSolve& s, const De
     size_t sm = 0;
     const void* k = p.staged ? pick_staged(p.rt, p.entry, p.deg, &sm) : pick_level(p.rt, p.entry, p.deg);
     if (!k) return cudaErrorInvalidValue;
-    return cudaLaunchKernel(k, dim3(p.grid), dim3(kWideThreads), args, p.smem, st);
+    return launch_pdl(k, dim3(p.grid), dim3(kWideThreads), args, p.smem, st);
 }
 
 cudaError_t launch_wide_decide(const DevSolve& s, const DevWide& w, int step, cudaStream_t st)
@@ -737,7 +809,26 @@ cudaError_t launch_wide_decide(const DevSolve& s, const DevWide& w, int step, cu
     DevWide c = w;
     int k = step;
     void* args[] = {&b, &c, &k};
-    return cudaLaunchKernel((const void*)wide_decide_kernel, dim3(1), dim3(kWideThreads), args, 0, st);
+    return launch_pdl((const void*)wide_decide_kernel, dim3(1), dim3(kWideThreads), args, 0, st);
+}
+
+bool wide_can_repack(const DevWide& w) { return w.rt > 1 && (int64_t)w.groups * w.rt <= kRepackSlots; }
+
+cudaError_t launch_wide_repack(const DevInstance& in, const DevSolve& s, const DevWide& w, const WidePlan& p,
+                               int32_t* tile_rep, cudaStream_t st)
+{
+    if (!wide_can_repack(w)) return cudaErrorInvalidValue;
+    wide_repack_plan_kernel<<<1, kWideThreads, 0, st>>>(w);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (p.rt == 4)
+        wide_repack_move_kernel<4><<<p.sms * 4, 512, 0, st>>>(in.n, w);
+    else
+        wide_repack_move_kernel<2><<<p.sms * 4, 512, 0, st>>>(in.n, w);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    wide_repack_swap_kernel<<<1, 256, 0, st>>>(w, tile_rep);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return launch_wide_decide(s, w, 0, st);  // the live groups anew
 }
 
 cudaError_t launch_wide_finalize(const DevInstance& in, const DevSolve& s, const DevWide& w, const WidePlan& p,

@@ -988,7 +988,7 @@ int mars_solve(mars_ctx* c, int32_t id, const mars_params* p, int8_t* best_spins
         ++launches;
     } else if (wide) {
         const float t0_max = *std::max_element(t0h.begin(), t0h.end());
-        if ((rc = run_sparse_wide(c, in->dev, p, s, wp, t0_max, S, &launches, &lvprof))) return rc;
+        if ((rc = run_sparse_wide(c, in->dev, p, s, wp, t0_max, dtile, S, &launches, &lvprof))) return rc;
         MARS_CUDA(c, cudaEventRecord(c->ev3, st));
     } else {
         if (sp.sell)

@@ -176,6 +176,13 @@ struct TcRun {
     // as a CUDA graph and replayed: 2P+2 launches become one graph launch.
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+    void drop_graph()
+    {
+        if (exec) cudaGraphExecDestroy(exec);
+        if (graph) cudaGraphDestroy(graph);
+        exec = nullptr;
+        graph = nullptr;
+    }
     // Replicas per warp in the chain, and the overlap of panel p+1's GEMM
     // with panel p's chain: the GEMMs run on `side`, the chains on the run's
     // stream, ordered by the events ev (fork, then per panel GEMM done and
@@ -214,8 +221,7 @@ struct TcRun {
     int32_t* flags = nullptr;
     ~TcRun()
     {
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
+        drop_graph();
         for (cudaEvent_t e : ev) cudaEventDestroy(e);
         if (side) cudaStreamDestroy(side);
     }
@@ -251,7 +257,8 @@ struct LevelProfile {
     int64_t launches = 0, updates = 0;
 };
 int run_sparse_wide(mars_ctx* c, const DevInstance& d, const mars_params* p, const DevSolve& s,
-                    const WidePlan& wp, float t0_max, Scratch& S, int64_t* launches, LevelProfile* prof);
+                    const WidePlan& wp, float t0_max, int32_t* tile_rep, Scratch& S, int64_t* launches,
+                    LevelProfile* prof);
 
 // Round-to-nearest-even FP32 -> BF16 bits (host side, for uploads).
 uint16_t float_to_bf16_bits(float f);

@@ -226,7 +226,8 @@ struct DevWide {
     int32_t* capped = nullptr;
     uint32_t* dmax = nullptr;        // the sweep's largest |change| (float bits, >= 0)
     int32_t* glist = nullptr;        // live groups, ascending
-    int32_t* counters = nullptr;     // [0] live groups, [1] live replicas
+    int32_t* counters = nullptr;     // [0] live groups, [1] live replicas, [2] slot pairs of a repacking
+    int2* pairs = nullptr;           // per slot: (dead slot, live slot) to exchange
 };
 struct WidePlan {
     int rt = 4;
@@ -247,6 +248,11 @@ cudaError_t launch_wide_level(const DevInstance& in, const DevSolve& s, const De
 // step != 0: the stopping rule and cooling after a sweep; then the live-group
 // list and counts (step == 0: the list only).
 cudaError_t launch_wide_decide(const DevSolve& s, const DevWide& w, int step, cudaStream_t st);
+// Move the live replicas into as few groups as hold them (exchanging slots;
+// tile_rep is s.tile_rep's buffer) and list the live groups anew.
+bool wide_can_repack(const DevWide& w);
+cudaError_t launch_wide_repack(const DevInstance& in, const DevSolve& s, const DevWide& w, const WidePlan& p,
+                               int32_t* tile_rep, cudaStream_t st);
 cudaError_t launch_wide_finalize(const DevInstance& in, const DevSolve& s, const DevWide& w, const WidePlan& p,
                                  cudaStream_t st);
 SparsePlan plan_sparse(const DevInstance& in, int R, int jacobi, int device);

@@ -114,10 +114,7 @@ int tc_plan(mars_ctx* c, TcRun* run, int32_t active, int32_t prefix)
         q.P = run->P;
         // every replica group and every GEMM item has a CTA of its own
         if (q.n_chain >= 1 && q.n_gemm >= 1 && q.chain_items <= q.n_chain && tiles * q.splitk <= q.n_gemm) {
-            if (run->exec) cudaGraphExecDestroy(run->exec);
-            if (run->graph) cudaGraphDestroy(run->graph);
-            run->exec = nullptr;
-            run->graph = nullptr;
+            run->drop_graph();
             run->persist = true;
             run->rpw = prpw;
             run->overlap = true;
@@ -167,10 +164,7 @@ int tc_plan(mars_ctx* c, TcRun* run, int32_t active, int32_t prefix)
     if (run->exec && rpc == run->chain_rpc && rpw == run->rpw && ovl == run->overlap && pr == run->pair && splitk == run->splitk &&
         tiles == run->gemm_tiles && chain_slots == run->chain_slots && cw == run->chain_warps)
         return MARS_OK;
-    if (run->exec) cudaGraphExecDestroy(run->exec);
-    if (run->graph) cudaGraphDestroy(run->graph);
-    run->exec = nullptr;
-    run->graph = nullptr;
+    run->drop_graph();
     run->rpw = rpw;
     run->chain_warps = cw;
     run->chain_rpc = rpc;

@@ -12,7 +12,8 @@
 #include <cmath>
 
 int run_sparse_wide(mars_ctx* c, const DevInstance& d, const mars_params* p, const DevSolve& s,
-                    const WidePlan& wp, float t0_max, Scratch& S, int64_t* launches, LevelProfile* prof)
+                    const WidePlan& wp, float t0_max, int32_t* tile_rep, Scratch& S, int64_t* launches,
+                    LevelProfile* prof)
 {
     cudaStream_t st = c->stream;
     int rc;
@@ -31,7 +32,8 @@ int run_sparse_wide(mars_ctx* c, const DevInstance& d, const mars_params* p, con
     if ((rc = S.get(slots, &w.capped))) return rc;
     if ((rc = S.get(slots, &w.dmax))) return rc;
     if ((rc = S.get((size_t)wp.groups, &w.glist))) return rc;
-    if ((rc = S.get(2, &w.counters))) return rc;
+    if ((rc = S.get(4, &w.counters))) return rc;
+    if ((rc = S.get(slots, &w.pairs))) return rc;
     MARS_CUDA(c, launch_wide_init(d, s, w, wp, st));
     MARS_CUDA(c, launch_wide_decide(s, w, 0, st));
     *launches += 2;
@@ -43,11 +45,16 @@ int run_sparse_wide(mars_ctx* c, const DevInstance& d, const mars_params* p, con
 
     int32_t* h = nullptr;
     MARS_CUDA(c, cudaMallocHost((void**)&h, 2 * sizeof(int32_t)));
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    // one sweep, and kMulti sweeps, as graphs: with a graph per sweep its start
+    // and end cost a lone replica's sweep more than its levels do
+    const int kMulti = d.nlev <= 64 ? 8 : 1;  // an order with many levels has long sweeps, and large graphs
+    cudaGraph_t graph[2] = {nullptr, nullptr};
+    cudaGraphExec_t exec[2] = {nullptr, nullptr};
     auto cleanup = [&]() {
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
+        for (int q = 0; q < 2; ++q) {
+            if (exec[q]) cudaGraphExecDestroy(exec[q]);
+            if (graph[q]) cudaGraphDestroy(graph[q]);
+        }
         cudaFreeHost(h);
     };
     auto check = [&](cudaError_t e, const char* what) -> int {
@@ -60,21 +67,26 @@ int run_sparse_wide(mars_ctx* c, const DevInstance& d, const mars_params* p, con
         return rc;
     if ((rc = check(cudaStreamSynchronize(st), "descent start"))) return rc;
 
-    // one sweep: the levels in order, then the decision
-    if ((rc = check(cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed), "sweep capture"))) return rc;
-    cudaError_t le = cudaSuccess;
-    for (int l = 0; l < d.nlev && le == cudaSuccess; ++l) le = launch_wide_level(d, s, w, wp, l, st);
-    if (le == cudaSuccess) le = launch_wide_decide(s, w, 1, st);
-    const cudaError_t ce = cudaStreamEndCapture(st, &graph);
-    if ((rc = check(le, "level launch"))) return rc;
-    if ((rc = check(ce, "sweep capture"))) return rc;
-    if ((rc = check(cudaGraphInstantiate(&exec, graph, 0), "sweep graph"))) return rc;
+    // a sweep: the levels in order, then the decision
+    for (int q = 0; q < (kMulti > 1 ? 2 : 1); ++q) {
+        if ((rc = check(cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed), "sweep capture"))) return rc;
+        cudaError_t le = cudaSuccess;
+        for (int k = 0; k < (q ? kMulti : 1) && le == cudaSuccess; ++k) {
+            for (int l = 0; l < d.nlev && le == cudaSuccess; ++l) le = launch_wide_level(d, s, w, wp, l, st);
+            if (le == cudaSuccess) le = launch_wide_decide(s, w, 1, st);
+        }
+        const cudaError_t ce = cudaStreamEndCapture(st, &graph[q]);
+        if ((rc = check(le, "level launch"))) return rc;
+        if ((rc = check(ce, "sweep capture"))) return rc;
+        if ((rc = check(cudaGraphInstantiate(&exec[q], graph[q], 0), "sweep graph"))) return rc;
+    }
 
     while ((int)c->prof.size() < 2 * d.nlev) {
         cudaEvent_t e;
         if ((rc = check(cudaEventCreate(&e), "event"))) return rc;
         c->prof.push_back(e);
     }
+    const bool repack = wide_can_repack(w) && env_flag("MARS_WIDE_REPACK", 1) != 0;
     int64_t done = 0;
     int batch = 1;
     while (h[1] > 0) {
@@ -83,6 +95,14 @@ int run_sparse_wide(mars_ctx* c, const DevInstance& d, const mars_params* p, con
             return fail(c, MARS_EDEVICE, "descent exceeded its sweep bound");
         }
         const int64_t live = h[1];
+        // Repack when at least an eighth of the live groups would empty: an
+        // exchange moves about 64 bytes per spin of a replica, which the next
+        // few sweeps save (a group's sweep moves 12 bytes per spin and slot).
+        const int full = (h[1] + wp.rt - 1) / wp.rt;
+        if (repack && 8 * (h[0] - full) >= h[0]) {
+            if ((rc = check(launch_wide_repack(d, s, w, wp, tile_rep, st), "repacking"))) return rc;
+            *launches += 4;
+        }
         // the batch's first sweep, each level launch timed
         for (int l = 0; l < d.nlev; ++l) {
             if ((rc = check(cudaEventRecord(c->prof[2 * l], st), "event"))) return rc;
@@ -90,8 +110,11 @@ int run_sparse_wide(mars_ctx* c, const DevInstance& d, const mars_params* p, con
             if ((rc = check(cudaEventRecord(c->prof[2 * l + 1], st), "event"))) return rc;
         }
         if ((rc = check(launch_wide_decide(s, w, 1, st), "decision launch"))) return rc;
-        for (int b = 1; b < batch; ++b)
-            if ((rc = check(cudaGraphLaunch(exec, st), "sweep graph launch"))) return rc;
+        for (int b = 1; b < batch;) {
+            const int many = kMulti > 1 && batch - b >= kMulti ? 1 : 0;
+            if ((rc = check(cudaGraphLaunch(exec[many], st), "sweep graph launch"))) return rc;
+            b += many ? kMulti : 1;
+        }
         if ((rc = check(cudaMemcpyAsync(h, w.counters, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st),
                         "counter copy")))
             return rc;
