@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(kEThreads, 1) dense_energy_kernel(DevInstance 
 
 template <bool INT>
 cudaError_t launch_as(const DevInstance& in, const int8_t* spins, int32_t count, double* e, long long* e_i64,
-                      int32_t* status, int planes, cudaStream_t st)
+                      int32_t* status, int planes, cudaStream_t st, int max_cluster)
 {
     const size_t smem = 1024 + 2 * kBuffer<INT> + (size_t)kTile * kSpinLd + (size_t)planes * kTile * sizeof(long long) +
                         2 * sizeof(uint64_t);
@@ -422,14 +422,14 @@ cudaError_t launch_as(const DevInstance& in, const int8_t* spins, int32_t count,
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    // CTAs per vector group: the cluster size (up to 16, more than the portable
-    // 8) with the fewest waves per share of the tiles, the smaller one on a tie.
+    // CTAs per vector group: the cluster size (up to 16 where the GPU is this
+    // solve's alone, more than the portable 8) with the fewest waves per share of the tiles, the smaller one on a tie.
     // A cluster keeps inside one GPC, so the driver says how many fit at once.
     // n = 2048, 512 vectors: 0.41 ms with up to 8 CTAs, 0.23 ms with 16.
     const int groups = (count + kTile - 1) / kTile, T = in.n / kTile + 1;
     int cs = 1;
     long long cost = 0;
-    for (int c = 1; c <= 16 && (long long)c <= (long long)T * (T + 1) / 2; c *= 2) {
+    for (int c = 1; c <= max_cluster && (long long)c <= (long long)T * (T + 1) / 2; c *= 2) {
         attr[0].val.clusterDim.x = (unsigned)c;
         cfg.gridDim = dim3((unsigned)(groups * c));
         int fit = 0;
@@ -453,12 +453,12 @@ cudaError_t launch_as(const DevInstance& in, const int8_t* spins, int32_t count,
 }  // namespace
 
 cudaError_t launch_dense_energy(const DevInstance& in, const int8_t* spins, int32_t count, double* e,
-                                long long* e_i64, int32_t* status, cudaStream_t st)
+                                long long* e_i64, int32_t* status, cudaStream_t st, int max_cluster)
 {
     if (count <= 0) return cudaSuccess;
-    if (in.integer) return launch_as<true>(in, spins, count, e, e_i64, status, 1, st);
+    if (in.integer) return launch_as<true>(in, spins, count, e, e_i64, status, 1, st, max_cluster);
     const int planes = std::min(kMaxPlanes, std::max(1, (in.exact_bits + kDigit - 1) / kDigit));
-    return launch_as<false>(in, spins, count, e, e_i64, status, planes, st);
+    return launch_as<false>(in, spins, count, e, e_i64, status, planes, st, max_cluster);
 }
 
 }  // namespace mars

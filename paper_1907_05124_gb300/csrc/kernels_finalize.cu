@@ -155,10 +155,11 @@ cudaError_t launch_best(const DevSolve& s, int32_t n, int32_t integer, int8_t* b
 }
 
 cudaError_t launch_energy(const DevInstance& in, const int8_t* spins, int32_t count, double* e,
-                          long long* e_i64, int32_t* status, cudaStream_t st)
+                          long long* e_i64, int32_t* status, cudaStream_t st, int max_cluster)
 {
     if (count <= 0) return cudaSuccess;
-    if (in.dense && (in.integer || in.exact_ok)) return launch_dense_energy(in, spins, count, e, e_i64, status, st);
+    if (in.dense && (in.integer || in.exact_ok))
+        return launch_dense_energy(in, spins, count, e, e_i64, status, st, max_cluster);
     energy_kernel<<<count, kEnergyThreads, 0, st>>>(in, spins, e, e_i64, status);
     return cudaGetLastError();
 }

@@ -133,7 +133,7 @@ struct DevSolve {
     int8_t* best_out = nullptr;        // and the best replica's spins here
 };
 
-// One instance of a batched launch (kernels_sparse_sell.cu).
+// One instance of a batched launch (kernels_sparse_batch.cu).
 struct BatchJob {
     DevInstance in;
     DevSolve s;
@@ -417,11 +417,12 @@ inline bool energy_pass(const DevInstance& in, bool tc, int32_t R)
 }
 
 // Exact energies of dense instances with integer couplings or exact_ok
-// (kernels_dense_energy.cu); launch_energy routes them here.
+// (kernels_dense_energy.cu); launch_energy routes them here. A group of 128 vectors
+// takes a cluster of up to max_cluster CTAs, which start only together.
 cudaError_t launch_dense_energy(const DevInstance& in, const int8_t* spins, int32_t count, double* e,
-                                long long* e_i64, int32_t* status, cudaStream_t st);
+                                long long* e_i64, int32_t* status, cudaStream_t st, int max_cluster);
 cudaError_t launch_energy(const DevInstance& in, const int8_t* spins, int32_t count,
-                          double* e, long long* e_i64, int32_t* status, cudaStream_t st);
+                          double* e, long long* e_i64, int32_t* status, cudaStream_t st, int max_cluster = 16);
 
 // Read-only view of a context and one of its instances, for entry points that
 // live outside mars_api.cu (mars_noalloc.cu).

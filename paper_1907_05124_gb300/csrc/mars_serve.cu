@@ -326,11 +326,17 @@ int serve_copy_results(mars_ctx* c, ServeReq* q)
     return MARS_OK;
 }
 
+// Served energies take clusters of at most 4 CTAs: a cluster starts only when one
+// GPC has that many SMs free, and the persistent sparse launches may hold about
+// half of each GPC's (up to 20) for as long as sparse work lasts.
+constexpr int kServeEnergyCluster = 4;
+
 int serve_finish_enqueue(mars_ctx* c, ServeReq* q)
 {
     cudaStream_t st = q->st;
     if (energy_pass(q->dev, q->tc != nullptr, q->s.R))
-        MARS_CUDA(c, launch_energy(q->dev, q->s.sigma, q->s.R, q->s.energy, q->s.energy_i64, q->s.status, st));
+        MARS_CUDA(c, launch_energy(q->dev, q->s.sigma, q->s.R, q->s.energy, q->s.energy_i64, q->s.status, st,
+                                   kServeEnergyCluster));
     MARS_CUDA(c, launch_best(q->s, q->dev.n, q->dev.integer, q->dbest, q->dres, st));
     return serve_copy_results(c, q);
 }
