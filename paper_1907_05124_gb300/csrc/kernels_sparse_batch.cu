@@ -84,9 +84,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) sparse_sell_batch_kernel(const 
 // ring, oldest first; when none is left, thread 0 polls the ring's tail
 // (about 2 us apart, at most idle_polls times) and the CTA exits when nothing
 // new arrives. Descriptors written by the host's copies are read through
-// volatile loads (past L1), after the tail that published them.
+// volatile loads (past L1), after the tail that published them. Several launches
+// may work on one ring: a CTA inside a long replica outlives the others' idle
+// time, and the host replaces those (serve_ring_ensure_kernel).
 template <int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) serve_ring_kernel(ServeRing* ring, int idle_polls)
+__global__ void __launch_bounds__(NT, 1024 / NT) serve_ring_kernel(ServeRing* ring, int idle_polls, int32_t* passed,
+                                                                  int32_t* gone)
 {
     extern __shared__ __align__(16) float m[];
     __shared__ SlotState<2, NT / 32> S;
@@ -105,6 +108,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) serve_ring_kernel(ServeRing* ri
                     const int R = *reinterpret_cast<volatile int*>(&ring->jobs[k].s.R);
                     if (taken < R) break;
                     atomicMax(&ring->cursor, c + 1);
+                    *reinterpret_cast<volatile int*>(passed + k) = 1;
                     ++c;
                 }
                 if (c < tail) {
@@ -129,6 +133,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) serve_ring_kernel(ServeRing* ri
         run_batch_job<NT>(s_jobcopy, m, S);
         __syncthreads();
     }
+    if (threadIdx.x == 0) *reinterpret_cast<volatile int*>(gone + blockIdx.x) = 1;
 }
 
 }  // namespace
@@ -222,14 +227,15 @@ int ring_job_format(const DevInstance& in, const RingPlan& p, int* rt)
     return in.sell_pm1 ? 1 : 0;
 }
 
-cudaError_t launch_serve_ring(ServeRing* ring, const RingPlan& p, int idle_polls, cudaStream_t st)
+cudaError_t launch_serve_ring(ServeRing* ring, const RingPlan& p, int ctas, int idle_polls, int32_t* passed,
+                              int32_t* gone, cudaStream_t st)
 {
     if (p.threads != 1024) return cudaErrorInvalidValue;
     const void* k = (const void*)serve_ring_kernel<1024>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return e;
-    void* args[] = {(void*)&ring, (void*)&idle_polls};
-    return cudaLaunchKernel(k, dim3(p.grid), dim3(p.threads), args, p.smem, st);
+    void* args[] = {(void*)&ring, (void*)&idle_polls, (void*)&passed, (void*)&gone};
+    return cudaLaunchKernel(k, dim3(ctas), dim3(p.threads), args, p.smem, st);
 }
 
 }  // namespace mars

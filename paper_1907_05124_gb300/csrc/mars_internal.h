@@ -173,9 +173,12 @@ bool plan_serve_ring(int device, RingPlan* p);
 // width, 2 when two replicas' magnetisations fit, else 1), or -1 when the
 // job's magnetisations do not fit on chip.
 int ring_job_format(const DevInstance& in, const RingPlan& p, int* rt);
-// Persistent serving kernel: runs published jobs and exits after about
-// idle_polls x 2 us without new work (or when ring->stop is set).
-cudaError_t launch_serve_ring(ServeRing* ring, const RingPlan& p, int idle_polls, cudaStream_t st);
+// `ctas` CTAs of the persistent serving kernel: each runs published jobs and
+// exits after about idle_polls x 2 us without new work (or when ring->stop is
+// set). Host-mapped words tell the host what they did: passed[k] = 1 when every
+// replica of the job in slot k is taken, gone[b] = 1 when CTA b has exited.
+cudaError_t launch_serve_ring(ServeRing* ring, const RingPlan& p, int ctas, int idle_polls, int32_t* passed,
+                              int32_t* gone, cudaStream_t st);
 
 struct BatchPlan {
     int rt = 1;

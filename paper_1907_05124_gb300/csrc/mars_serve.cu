@@ -52,6 +52,16 @@ struct ServeReq {
     bool cancelled = false; // mars_cancel while it ran: discard its results at the end
 };
 
+// One launch of the serving kernel, on a stream of its own.
+struct RingLaunch {
+    cudaStream_t st = nullptr;
+    cudaEvent_t ev = nullptr;
+    int ctas = 0;
+    bool live = false;
+};
+// Launches that may be alive at once (see serve_ring_ensure_kernel).
+constexpr int kRingLaunches = 8;
+
 struct Serve {
     std::vector<cudaStream_t> streams;
     std::vector<int> free_slots;
@@ -72,13 +82,15 @@ struct Serve {
     BatchJob* stage_jobs = nullptr; // pinned [kRingCap]
     RingSlot* stage_slots = nullptr;
     int32_t* stage_tail = nullptr;
-    int32_t* done = nullptr;        // host-mapped flags [kRingCap]
+    // host-mapped: done[kRingCap], passed[kRingCap] and per launch slot
+    // gone[plan.grid] (launch_serve_ring)
+    int32_t* done = nullptr;
     int32_t* done_dev = nullptr;
     int ring_refs = 0;              // requests that still read their ring slot
-    cudaStream_t pub_st = nullptr, ring_st = nullptr;
-    cudaEvent_t ring_ev = nullptr;
-    bool kernel_live = false;
+    cudaStream_t pub_st = nullptr;
+    std::vector<RingLaunch> launches;
     int64_t tail = 0;
+    int64_t open = 0;               // first job not known to have all its replicas taken
     int64_t ring_jobs = 0;          // jobs served through the ring
     int64_t stream_jobs = 0;        // jobs served on their own streams
     int idle_polls = 50;            // about 100 us without work before the kernel exits
@@ -135,6 +147,8 @@ int serve_sparse_grid(const Serve* sv, int grid)
 
 void serve_delete(Serve* sv) { delete sv; }
 
+size_t ring_flag_words(const Serve* sv) { return 2 * (size_t)kRingCap + (size_t)kRingLaunches * sv->plan.grid; }
+
 // Set the ring up on first use; false when it is unavailable (then every
 // request takes its own stream).
 bool serve_ring_init(mars_ctx* c, Serve* sv)
@@ -147,13 +161,12 @@ bool serve_ring_init(mars_ctx* c, Serve* sv)
               cudaMallocHost((void**)&sv->stage_jobs, sizeof(BatchJob) * kRingCap) == cudaSuccess &&
               cudaMallocHost((void**)&sv->stage_slots, sizeof(RingSlot) * kRingCap) == cudaSuccess &&
               cudaMallocHost((void**)&sv->stage_tail, sizeof(int32_t) * kRingCap) == cudaSuccess &&
-              cudaHostAlloc((void**)&sv->done, sizeof(int32_t) * kRingCap, cudaHostAllocMapped) == cudaSuccess &&
+              cudaHostAlloc((void**)&sv->done, ring_flag_words(sv) * sizeof(int32_t), cudaHostAllocMapped) ==
+                  cudaSuccess &&
               cudaHostGetDevicePointer((void**)&sv->done_dev, sv->done, 0) == cudaSuccess &&
               cudaStreamCreateWithFlags(&sv->pub_st, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&sv->ring_st, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&sv->ring_ev, cudaEventDisableTiming) == cudaSuccess &&
               cudaDeviceSynchronize() == cudaSuccess;
-    if (ok) std::memset(sv->done, 0, sizeof(int32_t) * kRingCap);
+    if (ok) std::memset(sv->done, 0, ring_flag_words(sv) * sizeof(int32_t));
     sv->ring_on = ok;
     return ok;
 }
@@ -164,7 +177,7 @@ void serve_ring_free(Serve* sv)
         int32_t one = 1;
         cudaMemcpyAsync(&sv->ring->stop, &one, sizeof one, cudaMemcpyHostToDevice, sv->pub_st);
         cudaStreamSynchronize(sv->pub_st);
-        cudaStreamSynchronize(sv->ring_st);
+        for (RingLaunch& q : sv->launches) cudaStreamSynchronize(q.st);
         cudaFree(sv->ring);
         sv->ring = nullptr;
     }
@@ -173,29 +186,73 @@ void serve_ring_free(Serve* sv)
     if (sv->stage_tail) cudaFreeHost(sv->stage_tail);
     if (sv->done) cudaFreeHost(sv->done);
     if (sv->pub_st) cudaStreamDestroy(sv->pub_st);
-    if (sv->ring_st) cudaStreamDestroy(sv->ring_st);
-    if (sv->ring_ev) cudaEventDestroy(sv->ring_ev);
+    for (RingLaunch& q : sv->launches) {
+        cudaStreamDestroy(q.st);
+        cudaEventDestroy(q.ev);
+    }
+    sv->launches.clear();
     sv->stage_jobs = nullptr;
     sv->stage_slots = nullptr;
     sv->stage_tail = nullptr;
     sv->done = nullptr;
-    sv->pub_st = sv->ring_st = nullptr;
-    sv->ring_ev = nullptr;
+    sv->pub_st = nullptr;
     sv->ring_on = false;
 }
 
-// Launch the serving kernel unless one is still running.
+// Which launches of the serving kernel still run; their CTAs that have not
+// exited are counted into *ctas.
+int serve_ring_alive(mars_ctx* c, Serve* sv, int* ctas)
+{
+    *ctas = 0;
+    for (size_t k = 0; k < sv->launches.size(); ++k) {
+        RingLaunch& q = sv->launches[k];
+        if (!q.live) continue;
+        const cudaError_t e = cudaEventQuery(q.ev);
+        if (e == cudaSuccess) {
+            q.live = false;
+            continue;
+        }
+        if (e != cudaErrorNotReady) return fail(c, MARS_EDEVICE, "serving kernel: %s", cudaGetErrorString(e));
+        const volatile int32_t* gone = sv->done + 2 * kRingCap + k * sv->plan.grid;
+        for (int b = 0; b < q.ctas; ++b) *ctas += gone[b] == 0;
+    }
+    return MARS_OK;
+}
+
+// Keep the serving kernel's CTAs at work while a published job has replicas to
+// take. CTAs exit one by one when they find none, but their launch ends only
+// with its last replica, which may take seconds: a job published meanwhile had
+// that replica's CTA alone, after the replica (16 mixed requests 0.2 to 1.0 s
+// instead of 0.06 to 0.1). So the CTAs that have gone are launched anew, on
+// another stream, once they are a quarter of the grid; a smaller gap is not
+// worth one of the kRingLaunches. With all of those alive, each by a CTA in its
+// last replica, a job waits for the first of them to end.
 int serve_ring_ensure_kernel(mars_ctx* c, Serve* sv)
 {
-    if (sv->kernel_live) {
-        const cudaError_t e = cudaEventQuery(sv->ring_ev);
-        if (e == cudaErrorNotReady) return MARS_OK;
-        if (e != cudaSuccess) return fail(c, MARS_EDEVICE, "serving kernel: %s", cudaGetErrorString(e));
-        sv->kernel_live = false;
+    int alive = 0;
+    if (const int rc = serve_ring_alive(c, sv, &alive)) return rc;
+    const volatile int32_t* passed = sv->done + kRingCap;
+    while (sv->open < sv->tail && passed[sv->open]) ++sv->open;
+    if (sv->open == sv->tail || 4 * alive > 3 * sv->plan.grid) return MARS_OK;
+    size_t k = 0;
+    while (k < sv->launches.size() && sv->launches[k].live) ++k;
+    if (k == kRingLaunches) return MARS_OK;
+    if (k == sv->launches.size()) {
+        RingLaunch q;
+        MARS_CUDA(c, cudaStreamCreateWithFlags(&q.st, cudaStreamNonBlocking));
+        const cudaError_t e = cudaEventCreateWithFlags(&q.ev, cudaEventDisableTiming);
+        if (e != cudaSuccess) cudaStreamDestroy(q.st);
+        MARS_CUDA(c, e);
+        sv->launches.push_back(q);
     }
-    MARS_CUDA(c, launch_serve_ring(sv->ring, sv->plan, sv->idle_polls, sv->ring_st));
-    MARS_CUDA(c, cudaEventRecord(sv->ring_ev, sv->ring_st));
-    sv->kernel_live = true;
+    RingLaunch& q = sv->launches[k];
+    q.ctas = sv->plan.grid - alive;
+    const size_t at = 2 * kRingCap + k * sv->plan.grid;
+    std::memset(sv->done + at, 0, q.ctas * sizeof(int32_t));
+    MARS_CUDA(c, launch_serve_ring(sv->ring, sv->plan, q.ctas, sv->idle_polls, sv->done_dev + kRingCap,
+                                   sv->done_dev + at, q.st));
+    MARS_CUDA(c, cudaEventRecord(q.ev, q.st));
+    q.live = true;
     return MARS_OK;
 }
 
@@ -593,8 +650,8 @@ void serve_progress(mars_ctx* c)
             q->slot = -1;
         }
     }
-    // a published job is always taken up: relaunch the serving kernel if it
-    // went idle and exited before the job's tail reached it
+    // a published job is always taken up: relaunch the serving kernel's CTAs
+    // that went idle and exited before the job's tail reached them
     if (ring_pending) {
         const int rc = serve_ring_ensure_kernel(c, sv);
         if (rc) {
@@ -604,13 +661,13 @@ void serve_progress(mars_ctx* c)
     }
     // reset the ring once its kernel has exited and no request reads a slot
     if (sv->ring && sv->tail > 0 && sv->ring_refs == 0) {
-        const bool live = sv->kernel_live && cudaEventQuery(sv->ring_ev) == cudaErrorNotReady;
-        if (!live) {
-            sv->kernel_live = false;
-            if (cudaMemsetAsync(sv->ring, 0, sizeof(ServeRing), sv->pub_st) == cudaSuccess) {
-                std::memset(sv->done, 0, sizeof(int32_t) * kRingCap);
-                sv->tail = 0;
-            }
+        int alive = 0;
+        bool live = serve_ring_alive(c, sv, &alive) != MARS_OK;
+        for (const RingLaunch& q : sv->launches) live = live || q.live;
+        if (!live && cudaMemsetAsync(sv->ring, 0, sizeof(ServeRing), sv->pub_st) == cudaSuccess) {
+            std::memset(sv->done, 0, 2 * sizeof(int32_t) * kRingCap);
+            sv->tail = 0;
+            sv->open = 0;
         }
     }
     // admit: serving-ring jobs (small sparse requests) whenever fewer than
