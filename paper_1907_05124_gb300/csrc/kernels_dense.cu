@@ -490,7 +490,23 @@ __global__ void __launch_bounds__((kDenseWarps + 1) * 32) dense_staged_kernel(De
 // of row buffers filled. With one warp per replica (the staged kernel above)
 // the same sweeps ran at one warp per scheduler: n = 1024, R = 512 took 1.09 us a
 // spin on a GB300, and 0.38 here; n = 4096, R = 256 4.6, and 0.49.
+//
+// A row's `full` barrier goes by its number modulo sync_barriers, a multiple of
+// the warps per replica, not by its buffer: a wait by parity is sound only for
+// one who has seen the barrier's fill before, and with that count the row before
+// on a barrier was the same warp's. (With one barrier per buffer it was another
+// warp's row whenever the buffers were no multiple of the warps: a warp could
+// take the barrier's last but one fill for its own, and with fewer buffers than
+// warps always did.)
 constexpr int kSyncWarps = 16;
+
+// At least one barrier per buffer, so that a barrier's last row has been read
+// before the producer arms it again.
+__host__ __device__ constexpr int sync_barriers(int stages, int reps)
+{
+    const int phases = kSyncWarps / reps;
+    return (stages + phases - 1) / phases * phases;
+}
 
 template <int REPS>
 __global__ void __launch_bounds__((kSyncWarps + 1) * 32) dense_sync_kernel(DevInstance in, DevSolve s, int stages)
@@ -505,15 +521,14 @@ __global__ void __launch_bounds__((kSyncWarps + 1) * 32) dense_sync_kernel(DevIn
     float* rows = smem;
     float* m = smem + (size_t)stages * rb + (size_t)rep * 2 * n;
     float* mn = m + n;
+    const int bars = sync_barriers(stages, REPS);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)stages * rb + (size_t)REPS * 2 * n);
-    uint64_t* empty = full + stages;
+    uint64_t* empty = full + bars;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + stages);
     __shared__ float s_d[REPS][kPhases];
     if (threadIdx.x == 0) {
-        for (int k = 0; k < stages; ++k) {
-            tc::mbar_init(&full[k], 1);
-            tc::mbar_init(&empty[k], REPS);  // the warps of the row's phase
-        }
+        for (int k = 0; k < bars; ++k) tc::mbar_init(&full[k], 1);
+        for (int k = 0; k < stages; ++k) tc::mbar_init(&empty[k], REPS);  // the warps of the row's phase
         *abort_flag = 0;
         tc::fence_barrier_init();
     }
@@ -526,41 +541,53 @@ __global__ void __launch_bounds__((kSyncWarps + 1) * 32) dense_sync_kernel(DevIn
         lv.start(s, r);
     }
     bool any = __syncthreads_or(lv.act) != 0;
-    int st = 0;       // stage of row 0 of the next sweep
-    uint32_t ph = 0;  // and its parity
+    int st = 0, fb = 0;         // buffer and `full` barrier of row 0 of the next sweep
+    uint32_t ph = 0, fp = 0;    // and their parities
     bool first = true;
     while (any) {
         float d = 0.f;
         if (!worker) {
             // the producer: rows 0 .. n - 1, each once its buffer's last row has
             // been read (the first `stages` rows find theirs empty)
-            int q = st;
+            int q = st, b = fb;
             uint32_t qp = ph;
             if (lane == 0) {
                 for (int a = 0; a < n; ++a) {
                     if (!(first && a < stages) && !stage_wait(&empty[q], qp ^ 1u, abort_flag, s.status)) break;
-                    load_row(rows + (size_t)q * rb, in.Jf, a, n, &full[q]);
+                    load_row(rows + (size_t)q * rb, in.Jf, a, n, &full[b]);
                     if (++q == stages) {
                         q = 0;
                         qp ^= 1u;
                     }
+                    if (++b == bars) b = 0;
                 }
             }
             __syncwarp();
         } else {
+            int q = (st + phase) % stages, b = fb + phase;
+            uint32_t bp = fp;
+            if (b >= bars) {
+                b -= bars;
+                bp ^= 1u;
+            }
             for (int a = phase; a < n; a += kPhases) {
-                const int use = st + a;  // buffers passed since stage 0 of parity ph
-                const int q = use % stages;
-                const uint32_t qp = ph ^ ((use / stages) & 1u);
-                if (!__all_sync(0xffffffffu, stage_wait(&full[q], qp, abort_flag, s.status))) break;
+                if (!__all_sync(0xffffffffu, stage_wait(&full[b], bp, abort_flag, s.status))) break;
                 if (lv.act)
                     sweep_spin<true>(in, s, lv, rows + (size_t)q * rb + row_shift(a, n), m, mn, a, n4, lane, d);
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&empty[q]);
+                q = (q + kPhases) % stages;
+                b += kPhases;
+                if (b >= bars) {
+                    b -= bars;
+                    bp ^= 1u;
+                }
             }
         }
         ph ^= ((st + n) / stages) & 1u;
         st = (st + n) % stages;
+        fp ^= ((fb + n) / bars) & 1u;
+        fb = (fb + n) % bars;
         first = false;
         __syncthreads();  // every row of the sweep has been read, every field written
         if (lv.act) {
@@ -616,7 +643,8 @@ DensePlan plan_dense(const DevInstance& in, int R, int jacobi, int device)
         // Rows under way: two per phase (16 kB at least) where they fit.
         const int reps = R >= 2 * sms ? 4 : R >= sms ? 2 : 1;
         auto bytes = [&](int stages) {
-            return ((size_t)stages * rb + (size_t)2 * reps * in.n) * sizeof(float) + 2 * stages * sizeof(uint64_t) + 16;
+            return ((size_t)stages * rb + (size_t)2 * reps * in.n) * sizeof(float) +
+                   (sync_barriers(stages, reps) + stages) * sizeof(uint64_t) + 16;
         };
         int stages = std::min(2 * kSyncWarps / reps, in.n);
         while (stages > 2 && bytes(stages) + 2048 > (size_t)optin) --stages;
