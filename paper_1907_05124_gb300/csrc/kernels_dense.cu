@@ -450,12 +450,13 @@ __global__ void __launch_bounds__((kDenseWarps + 1) * 32) dense_staged_kernel(De
         float d = 0.f;
         if (warp == kDenseWarps) {  // the producer: row a's buffer takes the row `stages` after it
             for (int a = 0; a < n; ++a) {
+                bool ok = false;
                 if (lane == 0 && stage_wait(&empty[st], ph, abort_flag, s.status)) {
                     const int next = a + stages < n ? a + stages : a + stages - n;
                     load_row(rows + (size_t)st * rb, in.Jf, next, n, &full[st]);
+                    ok = true;
                 }
-                __syncwarp();
-                if (*abort_flag) break;
+                if (!__shfl_sync(0xffffffffu, ok, 0)) break;
                 next_stage();
             }
         } else {
@@ -472,12 +473,10 @@ __global__ void __launch_bounds__((kDenseWarps + 1) * 32) dense_staged_kernel(De
         if (lv.act) lv.after_sweep(s, __shfl_sync(0xffffffffu, d, 0));  // lane 0's spins were kept
         any = __syncthreads_or(lv.act) != 0 && !*abort_flag;
     }
-    // the `stages` copies issued ahead of the last consumed row
-    if (threadIdx.x == 0 && !*abort_flag)
-        for (int k = 0; k < stages; ++k) {
-            const int q = st + k < stages ? st + k : st + k - stages;
-            if (!tc::mbar_wait(&full[q], st + k < stages ? ph : ph ^ 1u, s.status)) break;
-        }
+    // the last copy into each buffer: up to `stages` are ahead of the last row
+    // consumed, and after a timeout too none may land in an exited CTA's memory
+    if (warp == kDenseWarps && lane == 0)
+        for (int q = 0; q < stages; ++q) tc::mbar_wait(&full[q], q < st ? ph ^ 1u : ph, s.status);
     __syncthreads();
     if (live) finish_replica(in, s, r, m, lane, lv);
 }
@@ -552,7 +551,8 @@ __global__ void __launch_bounds__((kSyncWarps + 1) * 32) dense_sync_kernel(DevIn
             int q = st, b = fb;
             uint32_t qp = ph;
             if (lane == 0) {
-                for (int a = 0; a < n; ++a) {
+                int a = 0;
+                for (; a < n; ++a) {
                     if (!(first && a < stages) && !stage_wait(&empty[q], qp ^ 1u, abort_flag, s.status)) break;
                     load_row(rows + (size_t)q * rb, in.Jf, a, n, &full[b]);
                     if (++q == stages) {
@@ -561,6 +561,10 @@ __global__ void __launch_bounds__((kSyncWarps + 1) * 32) dense_sync_kernel(DevIn
                     }
                     if (++b == bars) b = 0;
                 }
+                // the last rows' copies: after a timeout nobody reads them, and
+                // none may land in an exited CTA's memory
+                for (int k = max(a - stages, 0); k < a; ++k)
+                    tc::mbar_wait(&full[(fb + k) % bars], fp ^ (uint32_t)((fb + k) / bars & 1), s.status);
             }
             __syncwarp();
         } else {
@@ -608,7 +612,7 @@ __global__ void __launch_bounds__((kSyncWarps + 1) * 32) dense_sync_kernel(DevIn
         }
         any = __syncthreads_or(lv.act) != 0 && any;
     }
-    // no copy is in flight: the producer's last row was read before the sweep ended
+    // no copy is in flight: every row of the sweep was read, or waited for
     if (live && phase == 0) finish_replica(in, s, r, m, lane, lv);
 }
 
