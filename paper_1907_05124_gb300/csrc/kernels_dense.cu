@@ -689,8 +689,7 @@ cudaError_t launch_dense(const DevInstance& in, const DevSolve& s, const DensePl
 {
     const void* k = pick(p, s.jacobi != 0);
     if (p.smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)p.smem);
+        cudaError_t e = allow_all_smem(k);
         if (e != cudaSuccess) return e;
     }
     DevInstance a = in;

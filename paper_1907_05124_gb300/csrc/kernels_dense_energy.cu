@@ -408,7 +408,7 @@ cudaError_t launch_as(const DevInstance& in, const int8_t* spins, int32_t count,
     const size_t smem = 1024 + 2 * kBuffer<INT> + (size_t)kTile * kSpinLd + (size_t)planes * kTile * sizeof(long long) +
                         2 * sizeof(uint64_t);
     const void* k = (const void*)dense_energy_kernel<INT>;
-    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = allow_all_smem(k);
     if (err != cudaSuccess) return err;
     err = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);  // clusters of 16
     if (err != cudaSuccess) return err;

@@ -252,7 +252,7 @@ SparsePlan plan_sparse(const DevInstance& in, int R, int jacobi, int device)
     p.smem = p.onchip ? (size_t)in.n * rt * sizeof(float) : 0;
     const void* k = pick_kernel(rt, p.onchip != 0, jacobi != 0);
     if (p.smem > 48 * 1024)
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+        allow_all_smem(k);
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads, p.smem);
     if (per_sm < 1) per_sm = 1;
@@ -268,8 +268,7 @@ cudaError_t launch_sparse(const DevInstance& in, const DevSolve& s, const Sparse
     const void* k = pick_kernel(p.rt, p.onchip != 0, s.jacobi != 0);
     if (!k) return cudaErrorInvalidValue;
     if (p.smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)p.smem);
+        cudaError_t e = allow_all_smem(k);
         if (e != cudaSuccess) return e;
     }
     DevInstance a = in;

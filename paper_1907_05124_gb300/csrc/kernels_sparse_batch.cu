@@ -180,7 +180,7 @@ bool plan_sparse_batch(const DevInstance* ins, const int* reps, int count, int d
     p->threads = nt;
     p->smem = smem;
     const void* k = pick_batch(nt);
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_all_smem(k);
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, nt, smem);
     p->grid = sms * std::max(per_sm, 1);
@@ -191,7 +191,7 @@ cudaError_t launch_sparse_batch(const BatchJob* jobs, int count, int* cursor, co
                                 cudaStream_t st)
 {
     const void* k = pick_batch(p.threads);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    cudaError_t e = allow_all_smem(k);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&jobs, (void*)&count, (void*)&cursor};
     return cudaLaunchKernel(k, dim3(p.grid), dim3(p.threads), args, p.smem, st);
@@ -206,8 +206,7 @@ bool plan_serve_ring(int device, RingPlan* p)
     p->threads = 1024;
     p->smem = (size_t)optin - 16 * 1024;  // static shared memory and slack
     const void* k = (const void*)serve_ring_kernel<1024>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->smem) != cudaSuccess)
-        return false;
+    if (allow_all_smem(k) != cudaSuccess) return false;
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, p->threads, p->smem);
     p->grid = sms * std::max(per_sm, 1);
@@ -232,7 +231,7 @@ cudaError_t launch_serve_ring(ServeRing* ring, const RingPlan& p, int ctas, int 
 {
     if (p.threads != 1024) return cudaErrorInvalidValue;
     const void* k = (const void*)serve_ring_kernel<1024>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    cudaError_t e = allow_all_smem(k);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&ring, (void*)&idle_polls, (void*)&passed, (void*)&gone};
     return cudaLaunchKernel(k, dim3(ctas), dim3(p.threads), args, p.smem, st);

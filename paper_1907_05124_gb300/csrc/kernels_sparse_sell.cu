@@ -159,7 +159,7 @@ bool plan_sparse_sell(const DevInstance& in, int R, int device, SparsePlan* p)
     p->deg = deg;
     const void* k = pick(rt, nt, fmt, deg);
     if (!k) return false;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->smem);
+    allow_all_smem(k);
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, nt, p->smem);
     if (per_sm < 1) per_sm = 1;
@@ -174,7 +174,7 @@ cudaError_t launch_sparse_sell(const DevInstance& in, const DevSolve& s, const S
 {
     const void* k = p.onchip ? pick(p.rt, p.threads, p.entry, p.deg) : pick_sell_slab(p.rt, p.entry, p.deg);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    cudaError_t e = allow_all_smem(k);
     if (e != cudaSuccess) return e;
     DevInstance a = in;
     DevSolve b = s;

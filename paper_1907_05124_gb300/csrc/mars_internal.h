@@ -8,6 +8,20 @@
 
 namespace mars {
 
+// Let kernel k take as much dynamic shared memory as its static part leaves. The
+// limit is one per process: were it set to the size that a launch needs, a
+// smaller call of another thread could lower it in between.
+inline cudaError_t allow_all_smem(const void* k)
+{
+    int dev = 0, optin = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
+}
+
 // Device-side status words (status[0]); MARS_OK when clean.
 enum DeviceStatus : int32_t { kDevOk = 0, kDevBadIndex = 1, kDevTimeout = 2 };
 
