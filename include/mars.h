@@ -412,7 +412,8 @@ int mars_device_check(mars_ctx* ctx, int32_t budget_us);
  * (count*n int8, entries +-1, caller labels). e (count doubles) receives the
  * energy rounded once to the nearest double; e_i64 (nullable) receives it as
  * an integer for integer instances. spins/e/e_i64 follow flags. Errors:
- * MARS_EINVAL (an entry not +-1), MARS_ENOTFOUND, MARS_EDEVICE.
+ * MARS_EINVAL (an entry not +-1), MARS_ENOTFOUND, MARS_ETIMEOUT (a wait inside the
+ * kernel gave up), MARS_EDEVICE.
  */
 int mars_energy(mars_ctx* ctx, int32_t inst, const int8_t* spins, int32_t count, double* e,
                 int64_t* e_i64, uint32_t flags);

@@ -1398,8 +1398,12 @@ int mars_energy(mars_ctx* c, int32_t id, const int8_t* spins, int32_t count, dou
         if (e_i64) MARS_CUDA(c, cudaMemcpyAsync(e_i64, dei, count * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     }
     MARS_CUDA(c, cudaStreamSynchronize(st));
-    if (hstatus != kDevOk) return fail(c, MARS_EINVAL, "spins must be +-1");
-    return MARS_OK;
+    switch (const int out = energy_status_rc(hstatus)) {
+    case MARS_OK: return MARS_OK;
+    case MARS_EINVAL: return fail(c, out, "spins must be +-1");
+    case MARS_ETIMEOUT: return fail(c, out, "the energy kernel gave up waiting");
+    default: return fail(c, out, "device status %d", hstatus);
+    }
 }
 
 int mars_draw_replicas(mars_ctx* c, uint64_t seed, uint32_t stream, int32_t r0, int32_t R,

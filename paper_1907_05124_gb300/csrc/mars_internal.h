@@ -1,6 +1,8 @@
 // Internal interfaces between the host runtime (mars_api.cu) and the kernels.
 #pragma once
 
+#include "device_status.h"
+
 #include <cstdint>
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -21,9 +23,6 @@ inline cudaError_t allow_all_smem(const void* k)
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
 }
-
-// Device-side status words (status[0]); MARS_OK when clean.
-enum DeviceStatus : int32_t { kDevOk = 0, kDevBadIndex = 1, kDevTimeout = 2 };
 
 // Instance data on the device, relabelled so that one sweep is "levels in
 // order, any order within a level": new label a has caller label new2old[a].
