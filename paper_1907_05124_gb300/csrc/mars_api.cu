@@ -1000,7 +1000,7 @@ int mars_solve(mars_ctx* c, int32_t id, const mars_params* p, int8_t* best_spins
     }
     launches += tcprof.launches;
     if (energy_pass(in->dev, tc, R)) {
-        MARS_CUDA(c, launch_energy(in->dev, s.sigma, R, s.energy, s.energy_i64, s.status, st));
+        MARS_CUDA(c, launch_energy(in->dev, s.sigma, R, s.energy, s.energy_i64, s.status, st, energy_cluster(c->device)));
         ++launches;
     }
     MARS_CUDA(c, cudaEventRecord(c->ev2, st));
@@ -1191,7 +1191,7 @@ int mars_solve_batch(mars_ctx* c, int32_t count, const int32_t* insts, const mar
     for (int32_t j = 0; j < count; ++j) {
         const DevSolve& s = jobs[j].s;
         if (energy_pass(dins[j], false, jobs[j].s.R)) {
-            MARS_CUDA(c, launch_energy(dins[j], s.sigma, s.R, s.energy, nullptr, s.status, st));
+            MARS_CUDA(c, launch_energy(dins[j], s.sigma, s.R, s.energy, nullptr, s.status, st, energy_cluster(c->device)));
             ++launches;
         }
         MARS_CUDA(c, launch_best(s, dins[j].n, dins[j].integer, dbest[j], dres[j], st));
@@ -1390,7 +1390,7 @@ int mars_energy(mars_ctx* c, int32_t id, const int8_t* spins, int32_t count, dou
         if ((rc = S.get(count, &de))) return rc;
         if (e_i64 && (rc = S.get(count, &dei))) return rc;
     }
-    MARS_CUDA(c, launch_energy(in->dev, dsp, count, de, dei, dstatus, st));
+    MARS_CUDA(c, launch_energy(in->dev, dsp, count, de, dei, dstatus, st, energy_cluster(c->device)));
     int32_t hstatus = 0;
     MARS_CUDA(c, cudaMemcpyAsync(&hstatus, dstatus, sizeof hstatus, cudaMemcpyDeviceToHost, st));
     if (!devp) {

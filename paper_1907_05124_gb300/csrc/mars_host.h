@@ -62,6 +62,8 @@ struct Instance {
 
 struct Serve;  // the serving engine's request table (mars_serve.cu)
 void serve_release(mars_ctx* c);
+// The most CTAs that an energy pass launched now may put into a cluster.
+int energy_cluster(int device);
 void serve_delete(Serve* sv);
 
 struct mars_ctx {

@@ -438,7 +438,7 @@ inline bool energy_pass(const DevInstance& in, bool tc, int32_t R)
 cudaError_t launch_dense_energy(const DevInstance& in, const int8_t* spins, int32_t count, double* e,
                                 long long* e_i64, int32_t* status, cudaStream_t st, int max_cluster);
 cudaError_t launch_energy(const DevInstance& in, const int8_t* spins, int32_t count,
-                          double* e, long long* e_i64, int32_t* status, cudaStream_t st, int max_cluster = 16);
+                          double* e, long long* e_i64, int32_t* status, cudaStream_t st, int max_cluster);
 
 // Read-only view of a context and one of its instances, for entry points that
 // live outside mars_api.cu (mars_noalloc.cu).

@@ -10,6 +10,7 @@
 #include <deque>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -61,6 +62,44 @@ struct RingLaunch {
 };
 // Launches that may be alive at once (see serve_ring_ensure_kernel).
 constexpr int kRingLaunches = 8;
+
+// Energies beside serving take clusters of at most 4 CTAs: a cluster starts only
+// when one GPC has that many SMs free, and the persistent sparse launches may hold
+// about half of each GPC's (up to 20) for as long as sparse work lasts. Alone, one of
+// 16 is the faster (kernels_dense_energy.cu).
+constexpr int kServeEnergyCluster = 4, kEnergyCluster = 16;
+
+// The persistent sparse launches of every context in the process, by the event
+// that follows each: the energies of one context meet the CTAs of another's.
+struct SparseWatch {
+    std::mutex mu;
+    std::vector<std::pair<int, cudaEvent_t>> live;  // device, event
+};
+
+SparseWatch& sparse_watch()
+{
+    static SparseWatch w;
+    return w;
+}
+
+// `ev` has been recorded behind a persistent sparse launch.
+void watch_add(int device, cudaEvent_t ev)
+{
+    SparseWatch& w = sparse_watch();
+    std::lock_guard<std::mutex> lock(w.mu);
+    const std::pair<int, cudaEvent_t> x(device, ev);
+    if (std::find(w.live.begin(), w.live.end(), x) == w.live.end()) w.live.push_back(x);
+}
+
+// `ev` is about to be destroyed.
+void watch_drop(cudaEvent_t ev)
+{
+    SparseWatch& w = sparse_watch();
+    std::lock_guard<std::mutex> lock(w.mu);
+    w.live.erase(std::remove_if(w.live.begin(), w.live.end(),
+                                [&](const std::pair<int, cudaEvent_t>& x) { return x.second == ev; }),
+                 w.live.end());
+}
 
 struct Serve {
     std::vector<cudaStream_t> streams;
@@ -187,6 +226,7 @@ void serve_ring_free(Serve* sv)
     if (sv->done) cudaFreeHost(sv->done);
     if (sv->pub_st) cudaStreamDestroy(sv->pub_st);
     for (RingLaunch& q : sv->launches) {
+        watch_drop(q.ev);
         cudaStreamDestroy(q.st);
         cudaEventDestroy(q.ev);
     }
@@ -252,6 +292,7 @@ int serve_ring_ensure_kernel(mars_ctx* c, Serve* sv)
     MARS_CUDA(c, launch_serve_ring(sv->ring, sv->plan, q.ctas, sv->idle_polls, sv->done_dev + kRingCap,
                                    sv->done_dev + at, q.st));
     MARS_CUDA(c, cudaEventRecord(q.ev, q.st));
+    watch_add(c->device, q.ev);
     q.live = true;
     return MARS_OK;
 }
@@ -327,6 +368,7 @@ void serve_free_req(mars_ctx* c, Serve* sv, ServeReq* q)
         q->pinned = nullptr;
     }
     if (q->ev) {
+        watch_drop(q->ev);
         cudaEventDestroy(q->ev);
         q->ev = nullptr;
     }
@@ -382,11 +424,6 @@ int serve_copy_results(mars_ctx* c, ServeReq* q)
     q->state = ReqState::Finishing;
     return MARS_OK;
 }
-
-// Served energies take clusters of at most 4 CTAs: a cluster starts only when one
-// GPC has that many SMs free, and the persistent sparse launches may hold about
-// half of each GPC's (up to 20) for as long as sparse work lasts.
-constexpr int kServeEnergyCluster = 4;
 
 int serve_finish_enqueue(mars_ctx* c, ServeReq* q)
 {
@@ -568,7 +605,9 @@ int serve_launch(mars_ctx* c, Serve* sv, ServeReq* q)
     } else {
         MARS_CUDA(c, launch_sparse(q->dev, s, sp, st));
     }
-    return serve_finish_enqueue(c, q);
+    if (const int rc2 = serve_finish_enqueue(c, q)) return rc2;
+    if (!q->dev.dense) watch_add(c->device, q->ev);
+    return MARS_OK;
 }
 
 void serve_mark_failed(mars_ctx* c, Serve* sv, ServeReq* q, int rc)
@@ -727,6 +766,20 @@ void serve_release(mars_ctx* c)
     c->serve.reset();
 }
 
+int energy_cluster(int device)
+{
+    SparseWatch& w = sparse_watch();
+    std::lock_guard<std::mutex> lock(w.mu);
+    for (size_t k = 0; k < w.live.size();) {
+        if (w.live[k].first != device) {
+            ++k;
+            continue;
+        }
+        if (cudaEventQuery(w.live[k].second) == cudaErrorNotReady) return kServeEnergyCluster;
+        w.live.erase(w.live.begin() + (std::ptrdiff_t)k);
+    }
+    return kEnergyCluster;
+}
 
 extern "C" {
 
