@@ -55,6 +55,7 @@ constexpr int kGroup = 4;             // digit planes made from one read of a ti
 constexpr int kOp = kTile * kStep * 2;  // bytes of one operand tile
 constexpr int kRun = 32;              // tiles of a row summed before they are weighted: D < 4096 x 127
 constexpr int kParts = kEThreads / kTile;  // threads that weight a vector's rows of a tile
+constexpr int kShortPass = 6;  // steps of a pass that takes no cluster (an integer instance below n = 256)
 constexpr int kSpinLd = 132;           // bytes of a vector's spins of a row tile in shared memory
 
 template <bool INT>
@@ -424,11 +425,14 @@ cudaError_t launch_as(const DevInstance& in, const int8_t* spins, int32_t count,
     cfg.numAttrs = 1;
     // CTAs per vector group: the cluster size (up to 16 where the GPU is this
     // solve's alone, more than the portable 8) with the fewest waves per share of the tiles, the smaller one on a tie.
-    // A cluster keeps inside one GPC, so the driver says how many fit at once.
+    // A cluster keeps inside one GPC, so the driver says how many fit at once. It
+    // takes 5 us to say so, which up to kShortPass steps would not win back.
     // n = 2048, 512 vectors: 0.41 ms with up to 8 CTAs, 0.23 ms with 16.
     const int groups = (count + kTile - 1) / kTile, T = in.n / kTile + 1;
+    const long long steps = (long long)T * (T + 1) * ((planes + kPlanesAtOnce<INT> - 1) / kPlanesAtOnce<INT>);
     int cs = 1;
     long long cost = 0;
+    if (T == 1 || steps <= kShortPass) max_cluster = 0;  // one CTA per group
     for (int c = 1; c <= max_cluster && (long long)c <= (long long)T * (T + 1) / 2; c *= 2) {
         attr[0].val.clusterDim.x = (unsigned)c;
         cfg.gridDim = dim3((unsigned)(groups * c));

@@ -38,9 +38,18 @@ __global__ void __launch_bounds__(kBestThreads) best_kernel(DevSolve s, int32_t 
 
 constexpr int kEnergyThreads = 256;
 
+// Dense instances up to this size take one CTA per vector, up to so many spins in all:
+// the tiled pass costs a cluster launch and up to 16 steps for the digits of a single
+// tile. mars_energy, us, one CTA per vector against tiled: n = 16 with 16 to 512
+// vectors 60 / 87 (Gaussian) and 54 / 63 (+-1), n = 64 with 512 85 / 89 and 63 / 64;
+// n = 16 with 4096 103 / 97 and 86 / 70, n = 64 with 4096 215 / 104 and 92 / 76.
+constexpr int kSmallEnergy = 64;
+constexpr int64_t kSmallSpins = 32768;
+
 // Energies of spin vectors, one CTA per vector: sparse instances, and dense
-// ones whose span exceeds the exact accumulator. Integer couplings sum exactly
-// in int64; other couplings sum exactly in an ExactAcc and are rounded once.
+// ones that are small (launch_energy) or whose span exceeds the exact accumulator.
+// Integer couplings sum exactly in int64; other couplings sum exactly in an ExactAcc
+// and are rounded once.
 __global__ void __launch_bounds__(kEnergyThreads) energy_kernel(DevInstance in, const int8_t* spins,
                                                                 double* e, long long* e_i64,
                                                                 int32_t* status)
@@ -59,9 +68,17 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_kernel(DevInstance in, 
     for (int a = tid; a < n; a += kEnergyThreads) {
         const int sa = sp[__ldg(in.new2old + a)];
         if (sa != 1 && sa != -1) { atomicExch(status, (int)kDevBadIndex); continue; }
-        if (in.dense) {  // the span exceeds the accumulator (launch_energy)
+        if (in.dense && in.integer) {
+            const int8_t* row = in.J_i8 + (size_t)a * n;
+            int acc = 0;
+            for (int b = a + 1; b < n; ++b) acc += (int)row[b] * (int)sp[__ldg(in.new2old + b)];
+            ei += acc * sa;  // n <= kSmallEnergy
+        } else if (in.dense) {
             const double* row = in.J_f64 + (size_t)a * n;
-            for (int b = a + 1; b < n; ++b) ef += sa * sp[__ldg(in.new2old + b)] > 0 ? row[b] : -row[b];
+            for (int b = a + 1; b < n; ++b) {
+                const double w = sa * sp[__ldg(in.new2old + b)] > 0 ? row[b] : -row[b];
+                if (exact) ex.add(w, in.exact_e0); else ef += w;
+            }
         } else {
             const int e0 = __ldg(in.row_ptr + a), e1 = __ldg(in.row_ptr + a + 1);
             if (in.integer) {
@@ -158,7 +175,8 @@ cudaError_t launch_energy(const DevInstance& in, const int8_t* spins, int32_t co
                           long long* e_i64, int32_t* status, cudaStream_t st, int max_cluster)
 {
     if (count <= 0) return cudaSuccess;
-    if (in.dense && (in.integer || in.exact_ok))
+    const bool small = in.n <= kSmallEnergy && (int64_t)in.n * count <= kSmallSpins;
+    if (in.dense && !small && (in.integer || in.exact_ok))
         return launch_dense_energy(in, spins, count, e, e_i64, status, st, max_cluster);
     energy_kernel<<<count, kEnergyThreads, 0, st>>>(in, spins, e, e_i64, status);
     return cudaGetLastError();
