@@ -355,13 +355,18 @@ void serve_free_req(mars_ctx* c, Serve* sv, ServeReq* q)
         sv->ring_refs -= 1;
         q->ring_job = -1;
     }
+    // A failed request may still have copies into its result block under way; a
+    // cancelled one is freed after its event, when they have ended. (Asked before the
+    // frees are queued: they would make the stream busy, and cudaFreeHost waits for
+    // the whole device.)
+    const bool copying = q->state == ReqState::Failed && q->rc != MARS_ECANCELED && q->st &&
+                         cudaStreamQuery(q->st) != cudaSuccess;
     if (q->st) {
         for (auto& b : q->bufs) dev_free_on(c, &b, q->st);
         q->bufs.clear();
     }
     if (q->pinned) {
-        // a failed request may still have copies into the block under way
-        if (q->state == ReqState::Failed && q->st && cudaStreamQuery(q->st) != cudaSuccess)
+        if (copying)
             cudaFreeHost(q->pinned);
         else
             pinned_put(sv, q->pinned, q->pinned_bytes);
