@@ -150,8 +150,8 @@ const void* pick_batch(int nt)
 // chip: six graphs and lattices of 64 to 512 replicas took 107 ms with two
 // slots each and 62 with one) and its coupling format; shared memory of the
 // most demanding job.
-bool plan_sparse_batch(const DevInstance* ins, const int* reps, int count, int device, BatchPlan* p, int* fmts,
-                       int* rts)
+bool plan_sparse_batch(const DevInstance* ins, const int* reps, const bool* even, int count, int device, BatchPlan* p,
+                       int* fmts, int* rts)
 {
     int sms = 1, optin = 48 * 1024;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
@@ -165,7 +165,7 @@ bool plan_sparse_batch(const DevInstance* ins, const int* reps, int count, int d
     for (int j = 0; j < count; ++j) {
         const DevInstance& in = ins[j];
         if (in.dense || !in.slices || (!in.sell_pm1 && !in.sell_gen)) return false;
-        int rt = rt_set >= 0 ? (rt_set >= 2 ? 2 : 1) : few_replicas(in, reps[j], sms) ? 1 : 2;
+        int rt = rt_set >= 0 ? (rt_set >= 2 ? 2 : 1) : few_replicas(in, reps[j], sms, even[j]) ? 1 : 2;
         while (rt > 1 && m_bytes(in.n, rt) > budget) rt /= 2;
         if (m_bytes(in.n, rt) > budget) return false;
         const size_t table = half_table_bytes(in);

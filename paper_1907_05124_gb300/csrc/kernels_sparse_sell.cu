@@ -78,13 +78,15 @@ const void* pick(int rt, int nt, int fmt, int deg)
 
 // Launch shape: replica slots per CTA (RT) and threads per CTA.
 //
-// Slots: two amortise the coupling loads, one ends sooner: with few replicas
-// per SM a solve lasts as long as its longest replica, which two slots slow
-// down. Descents on a GB300, ms with one / two slots: R = 64 to 256 one is
-// faster on every lattice and graph tried (L = 32 R = 256 1.05 / 1.23, 3-D
-// L = 21 R = 256 8.4 / 10.3); R = 400, L = 100 5.4 / 6.1; R = 512, degree 12
-// 37.7 / 47.5, degree 40 47 / 37, L = 64 2.67 / 2.35; R = 1024, L = 100
-// 11.8 / 7.9.
+// Slots: two amortise the coupling loads, one ends sooner. A solve lasts as long as
+// its longest replica, which two slots slow down, until there are so many replicas,
+// or replicas so even (fixed sweeps, a low k_max), that it is bound by all of them.
+// Descents on a GB300, ms with one / two slots, k_max = 1000: 2-D L = 64, R = 320
+// 2.39 / 2.72, R = 512 2.69 / 2.87, R = 600 3.00 / 2.88; L = 100, R = 512 6.03 / 6.53;
+// 3-D L = 21, R = 320 10.4 / 12.9, R = 512 13.9 / 13.3; random graphs n = 20000 of
+// degree 6, R = 320 66 / 74, R = 512 79 / 76; degree 24, n = 5000, R = 320 85 / 100.
+// The degree-6 graph with k_max = 100: R = 320 9.4 / 10.4, R = 400 11.8 / 10.8,
+// R = 512 14.9 / 11.0; three fixed sweeps, R = 456: 0.70 / 0.52.
 //
 // Threads: no more than one per spin of the largest level. A sweep of a small
 // instance is a few hundred cycles per level, much of it the barrier over
@@ -94,7 +96,7 @@ const void* pick(int rt, int nt, int fmt, int deg)
 //
 // The instance's launch shape (mars_autotune, mars_set_shape), else
 // MARS_SELL_RT / MARS_SELL_THREADS / MARS_SELL_SMEM_TABLE, override both.
-bool plan_sparse_sell(const DevInstance& in, int R, int device, SparsePlan* p)
+bool plan_sparse_sell(const DevInstance& in, int R, int device, bool even, SparsePlan* p)
 {
     if (!in.slices || (!in.sell_pm1 && !in.sell_gen)) return false;
     int sms = 1, optin = 48 * 1024;
@@ -104,7 +106,7 @@ bool plan_sparse_sell(const DevInstance& in, int R, int device, SparsePlan* p)
     const LaunchShape& sh = in.shape;
     const int rt_set = sh.sell_rt >= 0 ? sh.sell_rt : env_int("MARS_SELL_RT", -1);
     const int nt_set = sh.sell_threads >= 0 ? sh.sell_threads : env_int("MARS_SELL_THREADS", -1);
-    int rt = rt_set >= 0 ? rt_set : few_replicas(in, R, sms) ? 1 : 2;
+    int rt = rt_set >= 0 ? rt_set : few_replicas(in, R, sms, even) ? 1 : 2;
     int nt = nt_set;
     if (nt < 0)
         for (nt = 128; nt < 1024 && nt < 32 * in.max_slices;) nt *= 2;

@@ -934,7 +934,7 @@ int mars_solve(mars_ctx* c, int32_t id, const mars_params* p, int8_t* best_spins
     } else if (tc) {
         rt = 1;
     } else {
-        if (s.jacobi || !plan_sparse_sell(in->dev, R, c->device, &sp))
+        if (s.jacobi || !plan_sparse_sell(in->dev, R, c->device, even_sweeps(p->fixed_sweeps, p->k_max), &sp))
             sp = plan_sparse(in->dev, R, s.jacobi, c->device);
         // Magnetisations beyond shared memory: every replica resident and each
         // level spread over the whole grid, when all of them fit in half of
@@ -1159,8 +1159,12 @@ int mars_solve_batch(mars_ctx* c, int32_t count, const int32_t* insts, const mar
     }
     BatchPlan bp;
     std::vector<int> fmts(count), rts(count), nrep(count);
-    for (int32_t j = 0; j < count; ++j) nrep[j] = params[j].replicas;
-    if (!plan_sparse_batch(dins.data(), nrep.data(), count, c->device, &bp, fmts.data(), rts.data()))
+    std::unique_ptr<bool[]> even(new bool[count]);
+    for (int32_t j = 0; j < count; ++j) {
+        nrep[j] = params[j].replicas;
+        even[j] = even_sweeps(params[j].fixed_sweeps, params[j].k_max);
+    }
+    if (!plan_sparse_batch(dins.data(), nrep.data(), even.get(), count, c->device, &bp, fmts.data(), rts.data()))
         return fail(c, MARS_EINVAL, "an instance is too large for the batched on-chip kernel");
     for (int32_t j = 0; j < count; ++j) {
         jobs[j].fmt = fmts[j];

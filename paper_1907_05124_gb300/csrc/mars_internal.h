@@ -199,8 +199,8 @@ struct BatchPlan {
     size_t smem = 0;
     int grid = 0;
 };
-bool plan_sparse_batch(const DevInstance* ins, const int* reps, int count, int device, BatchPlan* p, int* fmts,
-                       int* rts);
+bool plan_sparse_batch(const DevInstance* ins, const int* reps, const bool* even, int count, int device, BatchPlan* p,
+                       int* fmts, int* rts);
 cudaError_t launch_sparse_batch(const BatchJob* jobs, int count, int* cursor, const BatchPlan& p,
                                 cudaStream_t st);
 
@@ -218,7 +218,11 @@ struct SparsePlan {
     int entry = 0;      // its coupling format: 0 general, 1 +-1 words, 2 +-1 halfwords in smem
     int deg = 0;        // compile-time degree of a regular instance (4 or 6), else 0
 };
-bool plan_sparse_sell(const DevInstance& in, int R, int device, SparsePlan* p);
+bool plan_sparse_sell(const DevInstance& in, int R, int device, bool even, SparsePlan* p);
+// Whether the replicas of a solve take about as many sweeps each: fixed sweeps, or a
+// cap that cuts the long descents short. By default (k_max = 1000) the longest takes
+// several times the mean.
+inline bool even_sweeps(int fixed_sweeps, int k_max) { return fixed_sweeps > 0 || k_max < 1000; }
 // The sliced-ELL kernel with m in global-memory slabs (format 0 or 1, rt 1, 2
 // or 4); null for another combination.
 const void* pick_sell_slab(int rt, int fmt, int deg);

@@ -90,7 +90,7 @@ extern "C" int mars_solve_noalloc(mars_ctx* c, int32_t id, const mars_params* p,
         dp = plan_dense(in, R, 0, v.device);
         if (dp.scratch_floats) return noalloc_fail(c, MARS_EINVAL, "n too large for the on-chip dense path");
     } else {
-        if (!plan_sparse_sell(in, R, v.device, &sp)) sp = plan_sparse(in, R, 0, v.device);
+        if (!plan_sparse_sell(in, R, v.device, even_sweeps(p->fixed_sweeps, p->k_max), &sp)) sp = plan_sparse(in, R, 0, v.device);
         if (sp.scratch_floats) return noalloc_fail(c, MARS_EINVAL, "n too large for the on-chip sparse path");
         rt = sp.rt;
     }

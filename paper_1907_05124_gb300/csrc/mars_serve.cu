@@ -411,7 +411,7 @@ size_t serve_footprint(const DevInstance& d, const mars_params& p, int device)
     } else {
         // the serving ring needs no scratch; the stream route takes its plan's
         SparsePlan sp;
-        if (jacobi || !plan_sparse_sell(d, (int)R, device, &sp)) sp = plan_sparse(d, (int)R, jacobi ? 1 : 0, device);
+        if (jacobi || !plan_sparse_sell(d, (int)R, device, even_sweeps(p.fixed_sweeps, p.k_max), &sp)) sp = plan_sparse(d, (int)R, jacobi ? 1 : 0, device);
         b += sp.scratch_floats * sizeof(float);
     }
     return b;
@@ -571,7 +571,7 @@ int serve_launch(mars_ctx* c, Serve* sv, ServeReq* q)
             q->state = ReqState::RingRunning;
             return serve_ring_ensure_kernel(c, sv);
         }
-        if (s.jacobi || !plan_sparse_sell(q->dev, R, c->device, &sp))
+        if (s.jacobi || !plan_sparse_sell(q->dev, R, c->device, even_sweeps(p.fixed_sweeps, p.k_max), &sp))
             sp = plan_sparse(q->dev, R, s.jacobi, c->device);
         sp.grid = serve_sparse_grid(sv, sp.grid);  // the per-CTA buffers below follow the grid
         rt = sp.rt;
