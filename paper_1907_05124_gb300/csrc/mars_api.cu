@@ -1255,7 +1255,7 @@ int mars_set_shape(mars_ctx* c, int32_t id, const mars_shape* shape)
                 if (v == a) return true;
             return false;
         };
-        if (!in_set(shape->sell_rt, {1, 2, 4}) || !in_set(shape->sell_threads, {512, 1024}) ||
+        if (!in_set(shape->sell_rt, {1, 2, 4}) || !in_set(shape->sell_threads, {128, 256, 512, 1024}) ||
             !in_set(shape->sell_smem_table, {0, 1}) || !in_set(shape->tc_rpw, {1, 2, 4}) ||
             !in_set(shape->tc_overlap, {0, 1}) || !in_set(shape->tc_pair, {0, 1}))
             return fail(c, MARS_EINVAL, "launch shape value outside its allowed set");
@@ -1300,6 +1300,18 @@ int mars_autotune(mars_ctx* c, int32_t id, const mars_params* p, int32_t repeats
                 cands.push_back(sh);
             }
     } else if (!d.dense && p->update == MARS_UPDATE_GS && d.slices && (d.sell_pm1 || d.sell_gen)) {
+        // the library's own plan, written out, first: the others below need not hold
+        // it (CTAs of 128 and 256 threads)
+        DevInstance own = d;
+        own.shape = LaunchShape{};
+        SparsePlan sp;
+        if (plan_sparse_sell(own, p->replicas, c->device, even_sweeps(p->fixed_sweeps, p->k_max), &sp) && sp.onchip) {
+            LaunchShape sh;
+            sh.sell_rt = sp.rt;
+            sh.sell_threads = sp.threads;
+            sh.sell_smem_table = !d.sell16 || sp.entry == 2 ? 1 : 0;
+            cands.push_back(sh);
+        }
         for (int tab = 1; tab >= (d.sell16 ? 0 : 1); --tab)
             for (int nt : {1024, 512})
                 for (int rt : {1, 2, 4}) {
