@@ -92,7 +92,12 @@ const void* pick(int rt, int nt, int fmt, int deg)
 // instance is a few hundred cycles per level, much of it the barrier over
 // warps that had nothing to do. R = 64, L = 12, ms with 128 / 256 / 512 / 1024
 // threads: 0.274 / 0.286 / 0.321 / 0.394; R = 256, L = 32: 1.72 / 1.10 / 0.87 /
-// 1.05; L = 64, R = 320: 6.3 / 3.7 / 2.7 / 2.0.
+// 1.05; L = 64, R = 320: 6.3 / 3.7 / 2.7 / 2.0. General couplings are read through the
+// L1, which shrinks by the shared memory of every CTA the SM can hold: 1024 threads
+// instead of 512 leave room for a table of 192 kB (n = 2000, degree 12, R = 64 17.3 /
+// 9.7 ms, R = 320 25.8 / 13.2) and cost 1 % where it does not fit (degree 20, 56.0 /
+// 56.8); of 128 and 256 threads small instances have the use all the same (n = 1000,
+// degree 12, R = 64 7.3 ms with 256, 7.9 with 1024).
 //
 // The instance's launch shape (mars_autotune, mars_set_shape), else
 // MARS_SELL_RT / MARS_SELL_THREADS / MARS_SELL_SMEM_TABLE, override both.
@@ -110,6 +115,7 @@ bool plan_sparse_sell(const DevInstance& in, int R, int device, bool even, Spars
     int nt = nt_set;
     if (nt < 0)
         for (nt = 128; nt < 1024 && nt < 32 * in.max_slices;) nt *= 2;
+    if (nt_set < 0 && nt == 512 && !in.sell_pm1) nt = 1024;
     const int smem_table = sh.sell_smem_table >= 0 ? sh.sell_smem_table : env_int("MARS_SELL_SMEM_TABLE", 1);
     if (rt != 1 && rt != 2 && rt != 4) rt = 1;
     if (nt != 512 && nt != 1024 && nt != 256 && nt != 128) nt = 512;
