@@ -441,7 +441,7 @@ int mars_instance_dense(mars_ctx* c, int32_t n, const void* J, int32_t jt, const
     InstGuard guard{c, in.get()};
     if ((rc = check_order(c, order, n, &in->order))) return rc;
     const std::vector<int32_t>& o = in->order;  // new label a is caller spin o[a]
-    std::vector<float> Jf((size_t)n * n);
+    std::vector<float> Jf((size_t)n * n + 4);  // bulk copies of rows read whole 16-byte pieces
     std::vector<int8_t> Ji;
     std::vector<double> Jd;
     if (integer) Ji.resize((size_t)n * n); else Jd.resize((size_t)n * n);
@@ -509,7 +509,6 @@ int mars_instance_dense(mars_ctx* c, int32_t n, const void* J, int32_t jt, const
         if ((rc = upload(c, in.get(), Jsup, &d.Jsup))) return rc;
         if (!J8.empty() && (rc = upload(c, in.get(), J8, &d.J8))) return rc;
     }
-    Jf.resize(Jf.size() + 4, 0.f);  // bulk copies of rows read whole 16-byte pieces
     if ((rc = upload(c, in.get(), Jf, &d.Jf))) return rc;
     if ((rc = upload(c, in.get(), Ji, &d.J_i8))) return rc;
     if ((rc = upload(c, in.get(), Jd, &d.J_f64))) return rc;
