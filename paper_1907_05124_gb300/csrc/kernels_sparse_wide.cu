@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) wide_level_kernel(DevInstance
             typename V::T acc;
 #pragma unroll
             for (int k = 0; k < RT; ++k) V::set(acc, k, 0.f);
-            const int deg = DEG > 0 ? DEG : d.z;
+            const int deg = DEG > 0 ? DEG : in.sell16 ? d.z & 0xffff : d.z;  // with sell16 .z holds two numbers
 #pragma unroll 4
             for (int q = 0; q < deg; ++q) {
                 int c;
