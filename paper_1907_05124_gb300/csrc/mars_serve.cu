@@ -127,6 +127,7 @@ struct Serve {
     int32_t* done_dev = nullptr;
     int ring_refs = 0;              // requests that still read their ring slot
     cudaStream_t pub_st = nullptr;
+    cudaEvent_t reset_ev = nullptr; // behind the ring's last reset: a launch waits for it
     std::vector<RingLaunch> launches;
     int64_t tail = 0;
     int64_t open = 0;               // first job not known to have all its replicas taken
@@ -204,6 +205,7 @@ bool serve_ring_init(mars_ctx* c, Serve* sv)
                   cudaSuccess &&
               cudaHostGetDevicePointer((void**)&sv->done_dev, sv->done, 0) == cudaSuccess &&
               cudaStreamCreateWithFlags(&sv->pub_st, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreateWithFlags(&sv->reset_ev, cudaEventDisableTiming) == cudaSuccess &&
               cudaDeviceSynchronize() == cudaSuccess;
     if (ok) std::memset(sv->done, 0, ring_flag_words(sv) * sizeof(int32_t));
     sv->ring_on = ok;
@@ -225,6 +227,8 @@ void serve_ring_free(Serve* sv)
     if (sv->stage_tail) cudaFreeHost(sv->stage_tail);
     if (sv->done) cudaFreeHost(sv->done);
     if (sv->pub_st) cudaStreamDestroy(sv->pub_st);
+    if (sv->reset_ev) cudaEventDestroy(sv->reset_ev);
+    sv->reset_ev = nullptr;
     for (RingLaunch& q : sv->launches) {
         watch_drop(q.ev);
         cudaStreamDestroy(q.st);
@@ -289,6 +293,9 @@ int serve_ring_ensure_kernel(mars_ctx* c, Serve* sv)
     q.ctas = sv->plan.grid - alive;
     const size_t at = 2 * kRingCap + k * sv->plan.grid;
     std::memset(sv->done + at, 0, q.ctas * sizeof(int32_t));
+    // not before the ring's last reset has landed: a half-reset ring would show a job
+    // of before it
+    MARS_CUDA(c, cudaStreamWaitEvent(q.st, sv->reset_ev, 0));
     MARS_CUDA(c, launch_serve_ring(sv->ring, sv->plan, q.ctas, sv->idle_polls, sv->done_dev + kRingCap,
                                    sv->done_dev + at, q.st));
     MARS_CUDA(c, cudaEventRecord(q.ev, q.st));
@@ -708,7 +715,8 @@ void serve_progress(mars_ctx* c)
         int alive = 0;
         bool live = serve_ring_alive(c, sv, &alive) != MARS_OK;
         for (const RingLaunch& q : sv->launches) live = live || q.live;
-        if (!live && cudaMemsetAsync(sv->ring, 0, sizeof(ServeRing), sv->pub_st) == cudaSuccess) {
+        if (!live && cudaMemsetAsync(sv->ring, 0, sizeof(ServeRing), sv->pub_st) == cudaSuccess &&
+            cudaEventRecord(sv->reset_ev, sv->pub_st) == cudaSuccess) {
             std::memset(sv->done, 0, 2 * sizeof(int32_t) * kRingCap);
             sv->tail = 0;
             sv->open = 0;
