@@ -427,13 +427,15 @@ cudaError_t launch_best(const DevSolve& s, int32_t n, int32_t integer, int8_t* b
 // Whether the energies of a solve of R replicas come from launch_energy after
 // the descent: the exact sums of non-integer couplings, and dense integer
 // instances on the tensor-core path (`tc`) once the tiled pass beats the
-// finalize kernel's own sums. Those cost about 6e-13 s R n^2 on a GB300 (n =
-// 8192, R = 4096: 163 ms; the pass 5.7) and a serial walk along each row; the
-// pass never takes less than about 40 us.
+// finalize kernel's own sums. Those cost about 6e-13 s R n^2 on a GB300 and a
+// serial walk along each row, the pass about 30 us up to n = 512 and 1000
+// vectors. From the descent to the result, us, sums / pass: n = 512, R = 128 65 /
+// 63; n = 400, R = 252 68 / 62; n = 512, R = 252 77 / 62; n = 700, R = 64 94 / 62;
+// n = 8192, R = 4096 163,000 / 1,300.
 inline bool energy_pass(const DevInstance& in, bool tc, int32_t R)
 {
     if (!in.integer) return in.exact_ok != 0;
-    return in.dense && tc && (in.n > 512 || (double)R * in.n * in.n > 6.6e7);
+    return in.dense && tc && (in.n > 512 || (double)R * in.n * in.n > 4e7);
 }
 
 // Exact energies of dense instances with integer couplings or exact_ok

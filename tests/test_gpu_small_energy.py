@@ -38,3 +38,15 @@ def test_small_energies_are_the_oracles(ctx, family, n, count):
     with pytest.raises(mars.MarsError):
         ctx.energy(inst, s)
     ctx.free(inst)
+
+
+@pytest.mark.parametrize("R", [250, 251])
+def test_tensor_core_solves_on_both_sides_of_the_pass(ctx, R):
+    """Integer couplings, n = 400: the finalize kernel's sums up to 250 replicas, the
+    tiled pass (one launch more) beyond."""
+    J, _ = _couplings("pm1", 400, 7)
+    inst = ctx.add_dense(J)
+    r = ctx.solve(inst, R, 0.0, 40.0, c_step=20.0, fixed_sweeps=1, precision="bf16", seed=2,
+                  outputs=("energies", "spins"))
+    assert np.array_equal(r.energies, O.energies(O.Instance.dense(J), r.spins))
+    ctx.free(inst)
