@@ -21,10 +21,11 @@
 // last term into the tanh's argument exactly as chain_body does, so the results
 // are bit for bit chain_body's.
 //
-// What bounds it: issue on the chain's scheduler. The step alone (FMA, ex2, add,
-// rcp, FMA, select, FMA) takes 57 cycles; with the folds into the two runs at
-// hand 90, and a run's hand-over about 200, so a panel's steps take 15,000
-// cycles, and 18,000 where 32 replicas feed the next panel. chain_body keeps
+// What bounds it: issue on the chain's scheduler. By clock stamps (N = 8192) a step
+// takes 64 cycles in a panel's first run, which has no last run's values to fold
+// (FMA, ex2, add, rcp, FMA, select, FMA depend on one another), and about 86 in the
+// others; waiting for hand-overs takes 140 a run, so a panel's steps take 12,300 to
+// 12,800 cycles, and 15,700 where 32 replicas feed the next panel. chain_body keeps
 // 32 / RPW lanes on a replica, every one computing the step, so with all
 // replicas active two warps per scheduler issue about 260 cycles a step.
 // Measured on a GB300 at N = 8192, a sweep with 4096 replicas active: 1.96 ms

@@ -20,9 +20,10 @@
 // one vector group are dealt to the CTAs of a cluster, whose partial sums meet
 // in distributed shared memory, so the pass needs no scratch in device memory.
 //
-// What bounds it: the integer instructions that cut and place the digits (ALU
-// pipe 62 % busy and the tensor pipe 14 % with 16 warps; with 8 warps, or with
-// the loaded spins tested before the step, a third to a half slower).
+// What bounds it: the integer instructions that cut and place the digits, and the
+// barrier of every step (n = 4096, 2048 vectors: ALU pipe 52 % busy, an instruction
+// issued in 44 % of the cycles, barrier the first stall, tensor pipe 16 %; with 8
+// warps, or with the loaded spins tested before the step, a third to a half slower).
 // Measured on a GB300, FP32-valued Gaussian couplings (8 planes) and +-1:
 // n = 8192, 4096 vectors 7.6 and 1.3 ms; n = 2048, 512 vectors 0.23 and 0.07
 // ms. The byte-wise dp4a kernel this replaced (36 lanes a clock and SM) took

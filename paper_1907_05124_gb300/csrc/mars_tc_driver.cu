@@ -69,7 +69,8 @@ int tc_plan(mars_ctx* c, TcRun* run, int32_t active, int32_t prefix)
     const int A = run->adaptive && active > 0 ? active : run->t.R;
     int rpw, ov, pair;
     if (run->adaptive) {
-        // fastest all-active sweeps measured on a GB300 at N = 8192 (ms):
+        // fastest all-active sweeps measured on a GB300 at N = 8192 (ms), with
+        // chain_body's kernel (the split chain, below, is faster on both sides):
         // A = 4096 pairs/4 2.15; 2048 pairs/2 1.48; 1024 overlap/2 1.19;
         // 512 and below overlap/1 1.04-1.06
         rpw = A >= 3072 ? 4 : A >= 768 ? 2 : 1;
