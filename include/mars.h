@@ -302,7 +302,8 @@ int mars_solve_batch(mars_ctx* ctx, int32_t count, const int32_t* insts, const m
  * knob to the library's default (or to its MARS_* environment override).
  *   sell_rt          sparse sliced-ELL kernel: replica slots per CTA, 1|2|4
  *   sell_threads     threads per CTA, 128|256|512|1024 (128 and 256 run as 512
- *                    with four slots, or when the couplings are not on chip)
+ *                    with four slots, and where +-1 couplings are not held in
+ *                    shared memory)
  *   sell_smem_table  couplings staged in shared memory when they fit, 0|1
  *   tc_rpw           dense BF16 tensor-core descent: replicas per chain warp, 1|2|4
  *   tc_overlap       panel p+1's GEMM overlapped with panel p's chain, 0|1
@@ -327,12 +328,12 @@ int mars_get_shape(mars_ctx* ctx, int32_t inst, mars_shape* out);
  * Autotuner for batched execution (the launch shape is not in the paper).
  * Times every candidate shape of the path that params select (sparse
  * sliced-ELL: slots x threads x table placement; dense BF16: replicas per
- * warp x overlap), the library's own choice among them, on `repeats` blocking solves with params each, keeps the
- * fastest descent, stores that shape on the instance for later solves and
- * returns it in *best (nullable) with its time in *seconds (nullable). A
- * path with no choices times the default once per repeat. Blocking; the
- * caller's params drive every trial, so tune on a short schedule (e.g.
- * fixed_sweeps) when a full solve is long. Errors: as mars_solve, plus
+ * warp x overlap), the library's own choice among them, on `repeats` blocking
+ * solves with params each, keeps the fastest descent, stores that shape on the
+ * instance for later solves and returns it in *best (nullable) with its time in
+ * *seconds (nullable). A path with no choices times the default once per repeat.
+ * Blocking; the caller's params drive every trial, so tune on a short schedule
+ * (e.g. fixed_sweeps) when a full solve is long. Errors: as mars_solve, plus
  * MARS_EINVAL for repeats outside [1, 100]; on error the previous shape
  * stays.
  */
