@@ -542,6 +542,12 @@ __global__ void __launch_bounds__((kSyncWarps + 1) * 32) dense_sync_kernel(DevIn
     bool any = __syncthreads_or(lv.act) != 0;
     int st = 0, fb = 0;         // buffer and `full` barrier of row 0 of the next sweep
     uint32_t ph = 0, fp = 0;    // and their parities
+    // a sweep's turns through both, and a worker's way from row to row: no division
+    // inside the sweeps
+    const int n_st = n % stages, n_fb = n % bars, phase_st = phase % stages, step_st = kPhases % stages;
+    const uint32_t t_st = (uint32_t)(n / stages), t_fb = (uint32_t)(n / bars);
+    int issued = 0, fb0 = 0;    // the producer: the sweep's rows issued, and where they began
+    uint32_t fp0 = 0;
     bool first = true;
     while (any) {
         float d = 0.f;
@@ -550,26 +556,26 @@ __global__ void __launch_bounds__((kSyncWarps + 1) * 32) dense_sync_kernel(DevIn
             // been read (the first `stages` rows find theirs empty)
             int q = st, b = fb;
             uint32_t qp = ph;
+            fb0 = fb;
+            fp0 = fp;
+            issued = 0;
             if (lane == 0) {
-                int a = 0;
-                for (; a < n; ++a) {
+                for (int a = 0; a < n; ++a) {
                     if (!(first && a < stages) && !stage_wait(&empty[q], qp ^ 1u, abort_flag, s.status)) break;
                     load_row(rows + (size_t)q * rb, in.Jf, a, n, &full[b]);
+                    issued = a + 1;
                     if (++q == stages) {
                         q = 0;
                         qp ^= 1u;
                     }
                     if (++b == bars) b = 0;
                 }
-                // the last rows' copies: after a timeout nobody reads them, and
-                // none may land in an exited CTA's memory
-                for (int k = max(a - stages, 0); k < a; ++k)
-                    tc::mbar_wait(&full[(fb + k) % bars], fp ^ (uint32_t)((fb + k) / bars & 1), s.status);
             }
             __syncwarp();
         } else {
-            int q = (st + phase) % stages, b = fb + phase;
+            int q = st + phase_st, b = fb + phase;
             uint32_t bp = fp;
+            if (q >= stages) q -= stages;
             if (b >= bars) {
                 b -= bars;
                 bp ^= 1u;
@@ -580,7 +586,8 @@ __global__ void __launch_bounds__((kSyncWarps + 1) * 32) dense_sync_kernel(DevIn
                     sweep_spin<true>(in, s, lv, rows + (size_t)q * rb + row_shift(a, n), m, mn, a, n4, lane, d);
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&empty[q]);
-                q = (q + kPhases) % stages;
+                q += step_st;
+                if (q >= stages) q -= stages;
                 b += kPhases;
                 if (b >= bars) {
                     b -= bars;
@@ -588,10 +595,12 @@ __global__ void __launch_bounds__((kSyncWarps + 1) * 32) dense_sync_kernel(DevIn
                 }
             }
         }
-        ph ^= ((st + n) / stages) & 1u;
-        st = (st + n) % stages;
-        fp ^= ((fb + n) / bars) & 1u;
-        fb = (fb + n) % bars;
+        st += n_st;
+        ph ^= (t_st + (st >= stages)) & 1u;
+        if (st >= stages) st -= stages;
+        fb += n_fb;
+        fp ^= (t_fb + (fb >= bars)) & 1u;
+        if (fb >= bars) fb -= bars;
         first = false;
         __syncthreads();  // every row of the sweep has been read, every field written
         if (lv.act) {
@@ -612,7 +621,12 @@ __global__ void __launch_bounds__((kSyncWarps + 1) * 32) dense_sync_kernel(DevIn
         }
         any = __syncthreads_or(lv.act) != 0 && any;
     }
-    // no copy is in flight: every row of the sweep was read, or waited for
+    // No copy is in flight: every row of the last sweep was read. After a timeout it
+    // was not, and none may land in an exited CTA's memory.
+    if (warp == kSyncWarps && lane == 0 && *abort_flag)
+        for (int k = max(issued - stages, 0); k < issued; ++k)
+            tc::mbar_wait(&full[(fb0 + k) % bars], fp0 ^ (uint32_t)((fb0 + k) / bars & 1), s.status);
+    __syncthreads();
     if (live && phase == 0) finish_replica(in, s, r, m, lane, lv);
 }
 
