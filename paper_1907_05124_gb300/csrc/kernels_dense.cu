@@ -449,16 +449,14 @@ __global__ void __launch_bounds__((kDenseWarps + 1) * 32) dense_staged_kernel(De
     while (any) {
         float d = 0.f;
         if (warp == kDenseWarps) {  // the producer: row a's buffer takes the row `stages` after it
-            for (int a = 0; a < n; ++a) {
-                bool ok = false;
-                if (lane == 0 && stage_wait(&empty[st], ph, abort_flag, s.status)) {
+            if (lane == 0)  // whose st and ph alone follow
+                for (int a = 0; a < n; ++a) {
+                    if (!stage_wait(&empty[st], ph, abort_flag, s.status)) break;
                     const int next = a + stages < n ? a + stages : a + stages - n;
                     load_row(rows + (size_t)st * rb, in.Jf, next, n, &full[st]);
-                    ok = true;
+                    next_stage();
                 }
-                if (!__shfl_sync(0xffffffffu, ok, 0)) break;
-                next_stage();
-            }
+            __syncwarp();
         } else {
             for (int a = 0; a < n; ++a) {
                 if (!__all_sync(0xffffffffu, stage_wait(&full[st], ph, abort_flag, s.status))) break;
@@ -487,8 +485,8 @@ __global__ void __launch_bounds__((kDenseWarps + 1) * 32) dense_staged_kernel(De
 // rows ph, ph + 16 / REPS, ... of its replica, so a row is read from shared
 // memory by the REPS warps that need it, and a seventeenth warp keeps the ring
 // of row buffers filled. With one warp per replica (the staged kernel above)
-// the same sweeps ran at one warp per scheduler: n = 1024, R = 512 took 1.09 us a
-// spin on a GB300, and 0.38 here; n = 4096, R = 256 4.6, and 0.49.
+// the same sweeps ran at one warp per scheduler: n = 1024, R = 400 took 1.09 us a
+// spin on a GB300, and 0.36 here; n = 4096, R = 256 4.6, and 0.49.
 //
 // A row's `full` barrier goes by its number modulo sync_barriers, a multiple of
 // the warps per replica, not by its buffer: a wait by parity is sound only for
