@@ -628,6 +628,9 @@ __global__ void __launch_bounds__((kSyncWarps + 1) * 32) dense_sync_kernel(DevIn
     if (live && phase == 0) finish_replica(in, s, r, m, lane, lv);
 }
 
+// What the plan leaves of a block's shared memory (allow_smem).
+int keep_smem(const DensePlan& p) { return p.sync_reps ? 2048 : p.stages ? 0 : 4096; }
+
 const void* pick(const DensePlan& p, bool jacobi)
 {
     if (p.sync_reps)
@@ -701,7 +704,7 @@ cudaError_t launch_dense(const DevInstance& in, const DevSolve& s, const DensePl
 {
     const void* k = pick(p, s.jacobi != 0);
     if (p.smem > 48 * 1024) {
-        cudaError_t e = allow_all_smem(k);
+        cudaError_t e = allow_smem(k, keep_smem(p));
         if (e != cudaSuccess) return e;
     }
     DevInstance a = in;

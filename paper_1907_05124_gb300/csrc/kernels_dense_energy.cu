@@ -407,10 +407,14 @@ template <bool INT>
 cudaError_t launch_as(const DevInstance& in, const int8_t* spins, int32_t count, double* e, long long* e_i64,
                       int32_t* status, int planes, cudaStream_t st, int max_cluster)
 {
-    const size_t smem = 1024 + 2 * kBuffer<INT> + (size_t)kTile * kSpinLd + (size_t)planes * kTile * sizeof(long long) +
-                        2 * sizeof(uint64_t);
+    auto bytes = [](int np) {
+        return 1024 + 2 * kBuffer<INT> + (size_t)kTile * kSpinLd + (size_t)np * kTile * sizeof(long long) +
+               2 * sizeof(uint64_t);
+    };
+    const size_t smem = bytes(planes);
     const void* k = (const void*)dense_energy_kernel<INT>;
-    cudaError_t err = allow_all_smem(k);
+    // the limit is the process's: that of the largest pass, for every pass
+    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(kMaxPlanes));
     if (err != cudaSuccess) return err;
     err = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);  // clusters of 16
     if (err != cudaSuccess) return err;

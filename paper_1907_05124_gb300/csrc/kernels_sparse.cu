@@ -27,6 +27,7 @@ namespace mars {
 namespace {
 
 constexpr int kThreads = 512;
+constexpr int kKeepSmem = 8 * 1024;  // of a block's shared memory, for the static part (allow_smem)
 constexpr int kWarps = kThreads / 32;
 
 template <int RT, bool ONCHIP, bool JACOBI>
@@ -230,7 +231,7 @@ SparsePlan plan_sparse(const DevInstance& in, int R, int jacobi, int device)
     int sms = 1, optin = 48 * 1024;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
-    const size_t budget = (size_t)optin - 8 * 1024;  // leave room for static shared memory
+    const size_t budget = (size_t)optin - kKeepSmem;
     SparsePlan p;
     p.threads = kThreads;
     // Largest tile that still gives every SM at least one tile and fits on chip.
@@ -252,7 +253,7 @@ SparsePlan plan_sparse(const DevInstance& in, int R, int jacobi, int device)
     p.smem = p.onchip ? (size_t)in.n * rt * sizeof(float) : 0;
     const void* k = pick_kernel(rt, p.onchip != 0, jacobi != 0);
     if (p.smem > 48 * 1024)
-        allow_all_smem(k);
+        allow_smem(k, kKeepSmem);
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads, p.smem);
     if (per_sm < 1) per_sm = 1;
@@ -268,7 +269,7 @@ cudaError_t launch_sparse(const DevInstance& in, const DevSolve& s, const Sparse
     const void* k = pick_kernel(p.rt, p.onchip != 0, s.jacobi != 0);
     if (!k) return cudaErrorInvalidValue;
     if (p.smem > 48 * 1024) {
-        cudaError_t e = allow_all_smem(k);
+        cudaError_t e = allow_smem(k, kKeepSmem);
         if (e != cudaSuccess) return e;
     }
     DevInstance a = in;

@@ -10,6 +10,8 @@
 namespace mars {
 namespace {
 
+constexpr int kKeepSmem = 16 * 1024;  // of a block's shared memory, for the static part (allow_smem)
+
 // One job of a batched launch with its own slot width (1 or 2, job.rt),
 // coupling format and degree under the CTA's two-slot bookkeeping. Regular
 // instances of degree 4 or 6 (square and cubic lattices) have their coupling
@@ -156,7 +158,7 @@ bool plan_sparse_batch(const DevInstance* ins, const int* reps, const bool* even
     int sms = 1, optin = 48 * 1024;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
-    const size_t budget = (size_t)optin - 16 * 1024;
+    const size_t budget = (size_t)optin - kKeepSmem;
     const int rt_set = env_int("MARS_SELL_RT", -1);
     int nt = env_int("MARS_SELL_THREADS", 1024);
     if (nt != 512 && nt != 1024) nt = 1024;
@@ -180,7 +182,7 @@ bool plan_sparse_batch(const DevInstance* ins, const int* reps, const bool* even
     p->threads = nt;
     p->smem = smem;
     const void* k = pick_batch(nt);
-    allow_all_smem(k);
+    allow_smem(k, kKeepSmem);
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, nt, smem);
     p->grid = sms * std::max(per_sm, 1);
@@ -191,7 +193,7 @@ cudaError_t launch_sparse_batch(const BatchJob* jobs, int count, int* cursor, co
                                 cudaStream_t st)
 {
     const void* k = pick_batch(p.threads);
-    cudaError_t e = allow_all_smem(k);
+    cudaError_t e = allow_smem(k, kKeepSmem);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&jobs, (void*)&count, (void*)&cursor};
     return cudaLaunchKernel(k, dim3(p.grid), dim3(p.threads), args, p.smem, st);
@@ -204,9 +206,9 @@ bool plan_serve_ring(int device, RingPlan* p)
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     p->rt = 2;
     p->threads = 1024;
-    p->smem = (size_t)optin - 16 * 1024;  // static shared memory and slack
+    p->smem = (size_t)optin - kKeepSmem;
     const void* k = (const void*)serve_ring_kernel<1024>;
-    if (allow_all_smem(k) != cudaSuccess) return false;
+    if (allow_smem(k, kKeepSmem) != cudaSuccess) return false;
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, p->threads, p->smem);
     p->grid = sms * std::max(per_sm, 1);
@@ -231,7 +233,7 @@ cudaError_t launch_serve_ring(ServeRing* ring, const RingPlan& p, int ctas, int 
 {
     if (p.threads != 1024) return cudaErrorInvalidValue;
     const void* k = (const void*)serve_ring_kernel<1024>;
-    cudaError_t e = allow_all_smem(k);
+    cudaError_t e = allow_smem(k, kKeepSmem);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&ring, (void*)&idle_polls, (void*)&passed, (void*)&gone};
     return cudaLaunchKernel(k, dim3(ctas), dim3(p.threads), args, p.smem, st);

@@ -28,6 +28,8 @@
 namespace mars {
 namespace {
 
+constexpr int kKeepSmem = 12 * 1024;  // of a block's shared memory, for the static part (allow_smem)
+
 template <int RT, int NT, int FMT, int DEG>
 __global__ void __launch_bounds__(NT, 1024 / NT) sparse_sell_kernel(DevInstance in, DevSolve s)
 {
@@ -107,7 +109,7 @@ bool plan_sparse_sell(const DevInstance& in, int R, int device, bool even, Spars
     int sms = 1, optin = 48 * 1024;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
-    const size_t budget = (size_t)optin - 12 * 1024;  // static shared memory and slack
+    const size_t budget = (size_t)optin - kKeepSmem;
     const LaunchShape& sh = in.shape;
     const int rt_set = sh.sell_rt >= 0 ? sh.sell_rt : env_int("MARS_SELL_RT", -1);
     const int nt_set = sh.sell_threads >= 0 ? sh.sell_threads : env_int("MARS_SELL_THREADS", -1);
@@ -167,7 +169,7 @@ bool plan_sparse_sell(const DevInstance& in, int R, int device, bool even, Spars
     p->deg = deg;
     const void* k = pick(rt, nt, fmt, deg);
     if (!k) return false;
-    allow_all_smem(k);
+    allow_smem(k, kKeepSmem);
     int per_sm = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, nt, p->smem);
     if (per_sm < 1) per_sm = 1;
@@ -182,7 +184,7 @@ cudaError_t launch_sparse_sell(const DevInstance& in, const DevSolve& s, const S
 {
     const void* k = p.onchip ? pick(p.rt, p.threads, p.entry, p.deg) : pick_sell_slab(p.rt, p.entry, p.deg);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = allow_all_smem(k);
+    cudaError_t e = allow_smem(k, kKeepSmem);
     if (e != cudaSuccess) return e;
     DevInstance a = in;
     DevSolve b = s;
