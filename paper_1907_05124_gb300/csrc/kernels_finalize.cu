@@ -41,10 +41,11 @@ constexpr int kEnergyThreads = 256;
 // Dense instances up to this size take one CTA per vector, up to so many spins in all:
 // the tiled pass costs a cluster launch and up to 16 steps for the digits of a single
 // tile. mars_energy, us, one CTA per vector against tiled: n = 16 with 16 to 512
-// vectors 60 / 87 (Gaussian) and 54 / 63 (+-1), n = 64 with 512 85 / 89 and 63 / 64;
-// n = 16 with 4096 103 / 97 and 86 / 70, n = 64 with 4096 215 / 104 and 92 / 76.
+// vectors 60 / 87 (Gaussian) and 54 / 63 (+-1), n = 64 with 512 85 / 89 and 63 / 64,
+// n = 4 with 4096 73 / 75 and 70 / 58; n = 16 with 4096 103 / 97 and 86 / 70, n = 64
+// with 4096 215 / 104 and 92 / 76.
 constexpr int kSmallEnergy = 64;
-constexpr int64_t kSmallSpins = 32768;
+constexpr int64_t kSmallSpins = 32768, kSmallSpinsInt = 8192;
 
 // Energies of spin vectors, one CTA per vector: sparse instances, and dense
 // ones that are small (launch_energy) or whose span exceeds the exact accumulator.
@@ -175,7 +176,7 @@ cudaError_t launch_energy(const DevInstance& in, const int8_t* spins, int32_t co
                           long long* e_i64, int32_t* status, cudaStream_t st, int max_cluster)
 {
     if (count <= 0) return cudaSuccess;
-    const bool small = in.n <= kSmallEnergy && (int64_t)in.n * count <= kSmallSpins;
+    const bool small = in.n <= kSmallEnergy && (int64_t)in.n * count <= (in.integer ? kSmallSpinsInt : kSmallSpins);
     if (in.dense && !small && (in.integer || in.exact_ok))
         return launch_dense_energy(in, spins, count, e, e_i64, status, st, max_cluster);
     energy_kernel<<<count, kEnergyThreads, 0, st>>>(in, spins, e, e_i64, status);

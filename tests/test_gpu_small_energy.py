@@ -1,5 +1,5 @@
 """Energies of small dense instances, which take one CTA per vector up to 64 spins and
-32768 in all and the tiled pass beyond, and those of single-CTA tiled passes (integer
+32768 in all (8192 for integer couplings) and the tiled pass beyond, and those of single-CTA tiled passes (integer
 couplings below 256 spins): the oracle's exactly rounded sums, bit for bit."""
 import numpy as np
 import pytest
@@ -19,9 +19,8 @@ def ctx():
 
 
 @pytest.mark.parametrize("family", ["pm1", "int8", "f32", "wide", "subnormal"])
-@pytest.mark.parametrize("n,count", [(1, 5), (2, 1025), (31, 1057), (31, 1058), (63, 200), (64, 512),
-                                     (64, 513), (65, 7),
-                                     (126, 129), (128, 5), (254, 300), (255, 64)])
+@pytest.mark.parametrize("n,count", [(1, 5), (2, 1025), (31, 1057), (31, 1058), (63, 200), (64, 128),
+                                     (64, 129), (64, 512), (64, 513), (65, 7), (126, 129), (128, 5), (254, 300), (255, 64)])
 def test_small_energies_are_the_oracles(ctx, family, n, count):
     J, h = _couplings(family, n, n + count)
     h = h if n % 2 else None
