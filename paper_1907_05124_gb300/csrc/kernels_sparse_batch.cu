@@ -167,7 +167,7 @@ bool plan_sparse_batch(const DevInstance* ins, const int* reps, const bool* even
     for (int j = 0; j < count; ++j) {
         const DevInstance& in = ins[j];
         if (in.dense || !in.slices || (!in.sell_pm1 && !in.sell_gen)) return false;
-        int rt = rt_set >= 0 ? (rt_set >= 2 ? 2 : 1) : few_replicas(in, reps[j], sms, even[j]) ? 1 : 2;
+        int rt = rt_set >= 0 ? (rt_set >= 2 ? 2 : 1) : few_replicas(in, reps[j], sms, even[j], nt) ? 1 : 2;
         while (rt > 1 && m_bytes(in.n, rt) > budget) rt /= 2;
         if (m_bytes(in.n, rt) > budget) return false;
         const size_t table = half_table_bytes(in);

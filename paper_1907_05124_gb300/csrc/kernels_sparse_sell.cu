@@ -88,7 +88,10 @@ const void* pick(int rt, int nt, int fmt, int deg)
 // 3-D L = 21, R = 320 10.4 / 12.9, R = 512 13.9 / 13.3; random graphs n = 20000 of
 // degree 6, R = 320 66 / 74, R = 512 79 / 76; degree 24, n = 5000, R = 320 85 / 100.
 // The degree-6 graph with k_max = 100: R = 320 9.4 / 10.4, R = 400 11.8 / 10.8,
-// R = 512 14.9 / 11.0; three fixed sweeps, R = 456: 0.70 / 0.52.
+// R = 512 14.9 / 11.0; three fixed sweeps, R = 456: 0.70 / 0.52. Even replicas of small
+// instances are bound by latency as long as an SM has few threads at work: k_max = 100,
+// n = 301, degree 9, R = 512 (430 threads an SM) 1.56 / 1.64; n = 600, degree 6, R = 512
+// (860) 1.59 / 1.68; n = 2000, degree 12, R = 320 (1080) 3.34 / 3.16.
 //
 // Threads: no more than one per spin of the largest level. A sweep of a small
 // instance is a few hundred cycles per level, much of it the barrier over
@@ -113,11 +116,11 @@ bool plan_sparse_sell(const DevInstance& in, int R, int device, bool even, Spars
     const LaunchShape& sh = in.shape;
     const int rt_set = sh.sell_rt >= 0 ? sh.sell_rt : env_int("MARS_SELL_RT", -1);
     const int nt_set = sh.sell_threads >= 0 ? sh.sell_threads : env_int("MARS_SELL_THREADS", -1);
-    int rt = rt_set >= 0 ? rt_set : few_replicas(in, R, sms, even) ? 1 : 2;
     int nt = nt_set;
     if (nt < 0)
         for (nt = 128; nt < 1024 && nt < 32 * in.max_slices;) nt *= 2;
     if (nt_set < 0 && nt == 512 && !in.sell_pm1) nt = 1024;
+    int rt = rt_set >= 0 ? rt_set : few_replicas(in, R, sms, even, nt) ? 1 : 2;
     const int smem_table = sh.sell_smem_table >= 0 ? sh.sell_smem_table : env_int("MARS_SELL_SMEM_TABLE", 1);
     if (rt != 1 && rt != 2 && rt != 4) rt = 1;
     if (nt != 512 && nt != 1024 && nt != 256 && nt != 128) nt = 512;

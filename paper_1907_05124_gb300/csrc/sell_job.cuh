@@ -386,11 +386,13 @@ inline size_t half_table_bytes(const DevInstance& in)
     return (size_t)in.nslices * sizeof(int4) + (size_t)in.sell16_len * sizeof(uint32_t);
 }
 
-// Whether a solve of R replicas takes one slot per CTA (plan_sparse_sell); `even`:
-// its replicas take about as many sweeps each (even_sweeps).
-inline bool few_replicas(const DevInstance& in, int R, int sms, bool even)
+// Whether a solve of R replicas takes one slot per CTA of nt threads
+// (plan_sparse_sell); `even`: its replicas take about as many sweeps each
+// (even_sweeps), and then the threads at work on an SM decide.
+inline bool few_replicas(const DevInstance& in, int R, int sms, bool even, int nt)
 {
-    return R <= 2 * sms || (!even && 2 * R <= 7 * sms && in.nnz <= (int64_t)16 * in.n);
+    if (R <= 2 * sms) return true;
+    return (even ? (int64_t)R * nt <= (int64_t)960 * sms : 2 * R <= 7 * sms) && in.nnz <= (int64_t)16 * in.n;
 }
 
 inline int env_int(const char* name, int dflt)

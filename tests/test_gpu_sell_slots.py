@@ -17,10 +17,11 @@ def ctx():
         yield c
 
 
-@pytest.mark.parametrize("R,kw", [(456, dict(fixed_sweeps=3)), (456, dict(k_max=25)), (512, dict(k_max=100)),
-                                  (300, dict(k_max=100)), (320, dict())])
-def test_the_faster_slots(ctx, R, kw):
-    inst = ctx.add_csr(*I.er_graph(20000, 6, 4))
+@pytest.mark.parametrize("n,R,kw", [(20000, 456, dict(fixed_sweeps=3)), (20000, 456, dict(k_max=25)),
+                                    (20000, 512, dict(k_max=100)), (20000, 300, dict(k_max=100)),
+                                    (20000, 320, dict()), (600, 512, dict(k_max=100)), (2000, 512, dict(k_max=100))])
+def test_the_faster_slots(ctx, n, R, kw):
+    inst = ctx.add_csr(*I.er_graph(n, 6, 4))
 
     def fastest(**shape):
         ctx.set_shape(inst, **shape)
