@@ -360,7 +360,8 @@ __device__ __forceinline__ void load_row(float* buf, const float* J, int a, int 
     tc::bulk_load(buf, J + ((size_t)a * n - sh), bytes, full);
 }
 
-// Staged kernel: each row J[a,:] is fetched into shared memory once per CTA. With `stages` == n all of J stays there and every warp runs its
+// Staged kernel: each row J[a,:] is fetched into shared memory once per CTA.
+// RESIDENT (`stages` == n): all of J stays there and every warp runs its
 // replica's sweeps by itself. Otherwise the kDenseWarps replicas of a CTA sweep
 // the spins in lockstep and the rows pass through a ring of `stages` buffers,
 // filled by bulk copies (cp.async.bulk, completion on a `full` mbarrier per
@@ -377,7 +378,7 @@ __device__ __forceinline__ void load_row(float* buf, const float* J, int a, int 
 // GB300, ns: all of J on chip, n = 64, R = 256 305 (593 through the ring with a
 // replica's warp refilling it); ring, n = 256, R = 512 524 (695), n = 1024,
 // R = 256 826 (1080), n = 4096, R = 512 1967 (4682).
-template <bool JACOBI>
+template <bool JACOBI, bool RESIDENT>
 __global__ void __launch_bounds__((kDenseWarps + 1) * 32) dense_staged_kernel(DevInstance in, DevSolve s,
                                                                         int stages)
 {
@@ -387,13 +388,13 @@ __global__ void __launch_bounds__((kDenseWarps + 1) * 32) dense_staged_kernel(De
     const bool live = warp < kDenseWarps && r < s.R;
     const int n = in.n, n4 = (n & 3) == 0 ? n >> 2 : 0;
     const int per = n * (JACOBI ? 2 : 1), rb = row_floats(n);
-    const size_t jfloats = stages == n ? ((size_t)n * n + 3) & ~(size_t)3 : (size_t)stages * rb;
+    constexpr bool resident = RESIDENT;  // stages == n
+    const size_t jfloats = resident ? ((size_t)n * n + 3) & ~(size_t)3 : (size_t)stages * rb;
     float* rows = smem;
     float* m = smem + jfloats + (size_t)warp * per;
     float* mn = JACOBI ? m + n : m;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + jfloats + (size_t)kDenseWarps * per);
     uint64_t* empty = full + stages;
-    const bool resident = stages == n;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + stages);
 
     if (threadIdx.x == 0) {
@@ -421,7 +422,7 @@ __global__ void __launch_bounds__((kDenseWarps + 1) * 32) dense_staged_kernel(De
     }
     __syncwarp();
 
-    if (resident) {
+    if constexpr (resident) {
         const bool ok = stage_wait(&full[0], 0, abort_flag, s.status);
         if (__syncthreads_and(ok)) {
             while (lv.act) {
@@ -637,7 +638,10 @@ const void* pick(const DensePlan& p, bool jacobi)
         return p.sync_reps == 4 ? (const void*)dense_sync_kernel<4>
              : p.sync_reps == 2 ? (const void*)dense_sync_kernel<2>
                                 : (const void*)dense_sync_kernel<1>;
-    if (p.stages) return jacobi ? (const void*)dense_staged_kernel<true> : (const void*)dense_staged_kernel<false>;
+    if (p.stages && p.resident)
+        return jacobi ? (const void*)dense_staged_kernel<true, true> : (const void*)dense_staged_kernel<false, true>;
+    if (p.stages)
+        return jacobi ? (const void*)dense_staged_kernel<true, false> : (const void*)dense_staged_kernel<false, false>;
     if (p.onchip) return jacobi ? (const void*)dense_descent_kernel<true, true>
                                 : (const void*)dense_descent_kernel<true, false>;
     return jacobi ? (const void*)dense_descent_kernel<false, true>
@@ -688,6 +692,7 @@ DensePlan plan_dense(const DevInstance& in, int R, int jacobi, int device)
              --stages)
             if (bytes(stages) <= (size_t)optin) p.stages = stages;
         if (p.stages) {
+            p.resident = p.stages == in.n;
             p.smem = bytes(p.stages);
             p.threads = (kDenseWarps + 1) * 32;
         }

@@ -399,7 +399,8 @@ cudaError_t launch_tc_export(const TcState& t, const DevInstance& in, float* m_o
 struct DensePlan {
     int warps_per_block = 4;
     int threads = 128;
-    int stages = 0;  // > 0: the staged kernel with this many row buffers (n: all of J)
+    int stages = 0;  // > 0: the staged kernel with this many row buffers
+    bool resident = false;  // as many as rows: all of J
     int sync_reps = 0;  // > 0: the synchronous kernel with this many replicas per CTA
     int onchip = 1;
     size_t smem = 0;
